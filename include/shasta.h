@@ -195,7 +195,10 @@ shasta_status shasta_step(shasta_ctx* ctx, int nsteps);
 shasta_status shasta_sweep(shasta_ctx* ctx, int axis);
 
 /* Times the launch choices of the sweep kernels for this grid and keeps the
- * fastest per axis.  FP32 / MIXED: work range length and register variant (a
+ * fastest per axis.  FP32 / MIXED: the tiled sweep (short independent pieces
+ * of each line; the only choice on small grids; the environment may set
+ * SHASTA_TILE=off, or the number of a tile shape), or the streaming sweep with
+ * a work range length and register variant (a
  * sweep's positions, line groups of 32 lines x positions along the axis, are
  * cut into as many ranges as that length gives, handed to the resident warps;
  * the cuts balance each range's streaming cost, its cells plus a 13-position
@@ -208,8 +211,9 @@ shasta_status shasta_sweep(shasta_ctx* ctx, int axis);
  * state is unchanged; synchronous.  Errors: EINVAL (state not set), ECUDA. */
 shasta_status shasta_autotune(shasta_ctx* ctx);
 
-/* Current launch choice per axis: out[2a] = register variant (FP64: 0),
- * out[2a+1] = positions per work range (FP64: cells per line segment). */
+/* Current launch choice per axis: out[2a] = register variant (FP64, tiles: 0),
+ * out[2a+1] = positions per work range (FP64: cells per line segment; tiles:
+ * positions per tile). */
 shasta_status shasta_get_tuning(const shasta_ctx* ctx, int out[6]);
 
 /* Waits until all work enqueued on the context's stream has finished. */

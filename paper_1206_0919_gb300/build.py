@@ -47,6 +47,13 @@ UNITS = [
     ("sweep_fuse2.cu", FAST),
     ("sweep_mixed.cu", FAST),
     ("sweep_mixed64.cu", FAST),
+    ("tile_f32_ideal.cu", FAST),
+    ("tile_f32_bag.cu", FAST),
+    ("tile_f32_table.cu", FAST),
+    ("tile_mixed_ideal.cu", FAST),
+    ("tile_mixed_bag.cu", FAST),
+    ("tile_mixed64_ideal.cu", FAST),
+    ("tile_mixed64_bag.cu", FAST),
     ("batch_f32.cu", FAST),
     ("batch_mixed.cu", FAST),
     ("alu_peak.cu", FAST),

@@ -81,7 +81,13 @@ struct shasta_ctx {
   int wpb = 4;            // warps per block of the FP32 / MIXED kernels
   long long force_range = 0;  // nonzero: positions per work range (environment override)
   int force_variant = -1; // >= 0: launch variant (environment override)
+  // FP32 / MIXED: the tiled sweep of each axis (shape -1: none), and the
+  // environment's say (shape, or streaming only)
+  TilePlan tile[3] = {{-1, 0, 0, 0}, {-1, 0, 0, 0}, {-1, 0, 0, 0}};
+  int force_tile = -1;
+  bool stream_only = false;
   bool tuned = false;     // autotuned launch choice below is valid
+  bool tune_tile[3] = {false, false, false};
   int tune_var[3] = {0, 0, 0};
   long long tune_range[3] = {0, 0, 0};
   // FP32 / MIXED: per axis, the bounds of balanced work ranges (device), built
@@ -226,6 +232,14 @@ long long work_positions(const shasta_ctx* c, int axis) {
   return (plane + 31) / 32 * n;
 }
 
+// How one sweep runs: on tiles, or streamed with a register variant and a
+// work range length (FP64: cells per line segment).
+struct Choice {
+  bool tile;
+  int variant;
+  long long range;
+};
+
 // Range length giving every resident warp of one wave `share` ranges (at
 // least 24 positions: each piece pays a 13-position halo and lag).
 long long range_for(long long total, long long warps, double share) {
@@ -365,34 +379,89 @@ long long fp64_segment(const shasta_ctx* c, int axis) {
   return (n + nseg - 1) / nseg;
 }
 
+// Positions per resident warp of the streaming sweep along an axis.
+long long stream_share(const shasta_ctx* c, int axis) {
+  return work_positions(c, axis) / ((long long)c->sm_count * std::max(c->occ[c->eos.kind][axis][0], 1));
+}
+
+// Where the line lies between the tiled and the streaming sweep, by the
+// positions a resident warp would stream (its lead-in and lag are 13 more).
+// Tiles always below kTileAlways (128^3, 36 positions: 45 streaming, 33 us
+// tiled along y; 112^3, 24: 37 against 25); the untuned choice along y and z
+// changes at kTileShare (144^3, 51: 55.5 against 51.2; 160^3, 70: 65.1 against
+// 63.7; 176^3, 93: 78.0 against 85.2).  Along x, where streaming stages its
+// results through shared memory as well, tiles stay ahead (200^3, 137: 116
+// against 90; 256^3, 288: 211 against 197).  In between the autotuner times
+// both.
+constexpr long long kTileAlways = 40, kTileShare = 64;
+
 // Launch choice for an axis: environment overrides, else the autotuned
-// choice, else variant 0 and one range per resident warp (FP32 / MIXED) or
-// the default segment length (FP64).
-void launch_choice(const shasta_ctx* c, int axis, int& variant, long long& range) {
+// choice, else (FP32 / MIXED) tiles or variant 0 with one range per resident
+// warp by the rule above, (FP64) the default segment length.
+Choice launch_choice(const shasta_ctx* c, int axis) {
+  Choice h{false, 0, 0};
   if (c->o.precision == SHASTA_FP64) {
-    variant = 0;
-    range = c->tuned && c->tune_range[axis] > 0 ? c->tune_range[axis] : fp64_segment(c, axis);
-    if (c->force_range > 0) range = c->force_range;
-    return;
+    h.range = c->tuned && c->tune_range[axis] > 0 ? c->tune_range[axis] : fp64_segment(c, axis);
+    if (c->force_range > 0) h.range = c->force_range;
+    return h;
   }
-  variant = c->tuned ? c->tune_var[axis] : 0;
-  if (c->force_variant >= 0) variant = c->force_variant;
-  const long long warps = (long long)c->sm_count * c->occ[c->eos.kind][axis][variant];
-  range = c->tuned ? c->tune_range[axis] : range_for(work_positions(c, axis), warps, 1.0);
-  if (c->force_range > 0) range = c->force_range;
+  if (c->tile[axis].shape >= 0) {
+    h.tile = c->force_tile >= 0 || (c->tuned ? c->tune_tile[axis] : axis == 0 || stream_share(c, axis) < kTileShare);
+    if (h.tile) return h;
+  }
+  h.variant = c->tuned ? c->tune_var[axis] : 0;
+  if (c->force_variant >= 0) h.variant = c->force_variant;
+  const long long warps = (long long)c->sm_count * c->occ[c->eos.kind][axis][h.variant];
+  h.range = c->tuned ? c->tune_range[axis] : range_for(work_positions(c, axis), warps, 1.0);
+  if (c->force_range > 0) h.range = c->force_range;
+  return h;
 }
 
 // Balanced range tables for the current launch choice of every axis (before
 // launches or a capture).
 shasta_status prepare_ranges(shasta_ctx* c) {
   for (int axis = 0; axis < 3; ++axis) {
-    int v;
-    long long r;
-    launch_choice(c, axis, v, r);
-    const shasta_status st = ensure_ranges(c, axis, r, v);
+    const Choice h = launch_choice(c, axis);
+    if (h.tile) continue;
+    const shasta_status st = ensure_ranges(c, axis, h.range, h.variant);
     if (st != SHASTA_OK) return st;
   }
   return SHASTA_OK;
+}
+
+cudaError_t launch_tile(shasta_ctx* c, int axis, const SweepParams& P) {
+  const TilePlan& t = c->tile[axis];
+  const bool bag = c->eos.kind == SHASTA_EOS_BAG;
+  if (c->o.precision == SHASTA_MIXED)
+    return (bag ? launch_tile_mixed_bag : launch_tile_mixed_ideal)(P, t, axis, c->sm_count, c->stream);
+  if (c->o.precision == SHASTA_MIXED_FP64)
+    return (bag ? launch_tile_mixed64_bag : launch_tile_mixed64_ideal)(P, t, axis, c->sm_count, c->stream);
+  if (c->eos.kind == SHASTA_EOS_TABLE) return launch_tile_f32_table(P, t, axis, c->sm_count, c->stream);
+  return (bag ? launch_tile_f32_bag : launch_tile_f32_ideal)(P, t, axis, c->sm_count, c->stream);
+}
+
+// Cuts the lines of an axis into tiles and readies the kernel; leaves the
+// axis to the streaming sweep where there is no tiled one.
+cudaError_t plan_tiles(shasta_ctx* c, int axis) {
+  TilePlan& t = c->tile[axis];
+  t.shape = -1;
+  const long long n = axis == 0 ? c->g.nx : (axis == 1 ? c->g.ny : c->g.nz);
+  if (c->stream_only || n > kTileMaxLine || (long long)c->ncell / n >= (1LL << 31)) return cudaSuccess;
+  if (c->o.scheme == SHASTA_SCHEME_SPLIT) return cudaSuccess;
+  if (c->o.scheme == SHASTA_SCHEME_NO_ANTIFLUX && c->o.precision == SHASTA_FP32) return cudaSuccess;
+  int shape = tile_shape_for((int)n, axis);
+  if (c->force_tile >= 0 && (axis == 0 || kTileShapes[c->force_tile].xl == 2)) shape = c->force_tile;
+  const bool bag = c->eos.kind == SHASTA_EOS_BAG;
+  auto prep = c->o.precision == SHASTA_MIXED        ? (bag ? prepare_tile_mixed_bag : prepare_tile_mixed_ideal)
+              : c->o.precision == SHASTA_MIXED_FP64 ? (bag ? prepare_tile_mixed64_bag : prepare_tile_mixed64_ideal)
+              : c->eos.kind == SHASTA_EOS_TABLE     ? prepare_tile_f32_table
+                                                    : (bag ? prepare_tile_f32_bag : prepare_tile_f32_ideal);
+  const cudaError_t e = prep(axis, shape, &t.blocks_per_sm);
+  if (e != cudaSuccess) return e;
+  if (t.blocks_per_sm < 1) return cudaSuccess;
+  t.shape = shape;
+  tile_cut(t, (int)n);
+  return cudaSuccess;
 }
 
 cudaError_t launch_params(shasta_ctx* c, int axis, const SweepParams& P) {
@@ -409,10 +478,9 @@ cudaError_t launch_params(shasta_ctx* c, int axis, const SweepParams& P) {
 }
 
 cudaError_t launch_sweep(shasta_ctx* c, int axis) {
-  int variant;
-  long long range;
-  launch_choice(c, axis, variant, range);
-  cudaError_t e = launch_params(c, axis, sweep_params(c, axis, c->cur, variant, range));
+  const Choice h = launch_choice(c, axis);
+  const SweepParams P = sweep_params(c, axis, c->cur, h.variant, h.range);
+  cudaError_t e = h.tile ? launch_tile(c, axis, P) : launch_params(c, axis, P);
   if (e == cudaSuccess) c->cur ^= 1;
   return e;
 }
@@ -441,14 +509,16 @@ void drop_graph(shasta_ctx* c) {
   c->graph = nullptr;
 }
 
-// Mean time of `reps` sweeps of axis with parameters P (after `warm`
-// untimed ones), from the current buffer into the other one.
-cudaError_t time_choice(shasta_ctx* c, int axis, const SweepParams& P, int warm, int reps,
+// Time of `reps` sweeps of axis with parameters P, on tiles or streamed
+// (after `warm` untimed ones), from the current buffer into the other one.
+cudaError_t time_choice(shasta_ctx* c, int axis, bool tile, SweepParams P, int warm, int reps,
                         cudaEvent_t e0, cudaEvent_t e1, float& ms) {
+  P.clamp_count = nullptr;  // trial sweeps are no steps: their clamps do not count
+  auto go = [&] { return tile ? launch_tile(c, axis, P) : launch_params(c, axis, P); };
   cudaError_t ce = cudaSuccess;
-  for (int r = 0; r < warm && ce == cudaSuccess; ++r) ce = launch_params(c, axis, P);
+  for (int r = 0; r < warm && ce == cudaSuccess; ++r) ce = go();
   if (ce == cudaSuccess) ce = cudaEventRecord(e0, c->stream);
-  for (int r = 0; r < reps && ce == cudaSuccess; ++r) ce = launch_params(c, axis, P);
+  for (int r = 0; r < reps && ce == cudaSuccess; ++r) ce = go();
   if (ce == cudaSuccess) ce = cudaEventRecord(e1, c->stream);
   if (ce == cudaSuccess) ce = cudaEventSynchronize(e1);
   if (ce == cudaSuccess) ce = cudaEventElapsedTime(&ms, e0, e1);
@@ -457,8 +527,9 @@ cudaError_t time_choice(shasta_ctx* c, int axis, const SweepParams& P, int warm,
 
 // Times candidate launch choices per axis with repeated sweeps from the
 // current buffer into the other one (the state itself is not changed) and
-// keeps the fastest.  FP32 / MIXED: the register variant, and ranges of one
-// line group (no line is cut) or of 1/4 .. 3 ranges per resident warp.
+// keeps the fastest.  FP32 / MIXED: tiles (alone, untimed, where a warp's
+// streamed share is under kTileAlways), or the register variant and ranges of
+// one line group (no line is cut) or of 1/4 .. 3 ranges per resident warp.
 // FP64: the line segment length (the default one, 24 .. 128 cells, whole
 // lines).  The choice does not change results.
 shasta_status autotune(shasta_ctx* c) {
@@ -479,6 +550,19 @@ shasta_status autotune(shasta_ctx* c) {
     float best = 1e30f;
     int bv = 0;
     long long br = f64 ? fp64_segment(c, axis) : n;
+    bool bt = false;
+    if (c->tile[axis].shape >= 0) {
+      if (c->force_tile >= 0 || stream_share(c, axis) < kTileAlways) {
+        c->tune_tile[axis] = true;
+        continue;
+      }
+      const cudaError_t ce = time_choice(c, axis, true, sweep_params(c, axis, c->cur, 0, 1), 2, 4, e0, e1, best);
+      if (ce != cudaSuccess) {
+        st = cuda_fail(c, ce, "autotune");
+        break;
+      }
+      bt = true;
+    }
     for (int var = 0; var < (f64 ? 1 : 2); ++var) {
       long long cands[8];
       int nc = 0;
@@ -504,7 +588,7 @@ shasta_status autotune(shasta_ctx* c) {
         st = ensure_ranges(c, axis, cands[ci], var);
         if (st != SHASTA_OK) break;
         float ms = 0;
-        const cudaError_t ce = time_choice(c, axis, sweep_params(c, axis, c->cur, var, cands[ci]),
+        const cudaError_t ce = time_choice(c, axis, false, sweep_params(c, axis, c->cur, var, cands[ci]),
                                            f64 ? 1 : 2, f64 ? 2 : 4, e0, e1, ms);
         if (ce != cudaSuccess) {
           st = cuda_fail(c, ce, "autotune");
@@ -514,11 +598,14 @@ shasta_status autotune(shasta_ctx* c) {
           best = ms;
           bv = var;
           br = cands[ci];
+          bt = false;
         }
       }
     }
+    c->tune_tile[axis] = bt;
     c->tune_var[axis] = bv;
     c->tune_range[axis] = br;
+    if (bt) continue;
     // FP32 / MIXED: the work shares of the CTAs of an SM for that choice
     if (!f64 && st == SHASTA_OK && c->balance && c->force_range == 0 && !c->force_skew) {
       const double keep = c->rank_skew[axis];
@@ -529,7 +616,7 @@ shasta_status autotune(shasta_ctx* c) {
         st = ensure_ranges(c, axis, br, bv);
         if (st != SHASTA_OK) break;
         float ms = 0;
-        const cudaError_t ce = time_choice(c, axis, sweep_params(c, axis, c->cur, bv, br), 2, 4, e0, e1, ms);
+        const cudaError_t ce = time_choice(c, axis, false, sweep_params(c, axis, c->cur, bv, br), 2, 4, e0, e1, ms);
         if (ce != cudaSuccess) {
           st = cuda_fail(c, ce, "autotune");
           break;
@@ -702,6 +789,13 @@ shasta_status shasta_create(const shasta_grid* g, double dx, double lambda, cons
     }
     v = getenv("SHASTA_EDGE_COST");
     if (v && atof(v) >= 0.0 && atof(v) <= 64.0) c->edge_cost = atof(v);
+    // a forced choice of the streaming sweep leaves the tiles out
+    c->stream_only = c->force_range > 0 || !c->balance || c->force_variant >= 0 || c->force_skew || v;
+    v = getenv("SHASTA_TILE");
+    if (v && !strcmp(v, "off"))
+      c->stream_only = true;
+    else if (v && *v >= '0' && *v <= '9' && atoi(v) < kTileShapeCount)
+      c->force_tile = atoi(v);
   }
   auto bail = [&](cudaError_t err, const char* where) {
     std::string m = std::string(where) + ": " + cudaGetErrorString(err);
@@ -790,6 +884,10 @@ shasta_status shasta_create(const shasta_grid* g, double dx, double lambda, cons
     c->wpb = opts.precision == SHASTA_MIXED        ? sweep_warps_per_block_mixed()
              : opts.precision == SHASTA_MIXED_FP64 ? sweep_warps_per_block_mixed64()
                                                    : sweep_warps_per_block_f32();
+    for (int a = 0; a < 3; ++a) {
+      err = plan_tiles(c, a);
+      if (err != cudaSuccess) return bail(err, "prepare tiled sweep kernels");
+    }
   }
   if (opts.stream) {
     c->stream = (cudaStream_t)opts.stream;
@@ -917,10 +1015,9 @@ shasta_status shasta_autotune(shasta_ctx* c) {
 shasta_status shasta_get_tuning(const shasta_ctx* c, int out[6]) {
   if (!c || !out) return SHASTA_EINVAL;
   for (int a = 0; a < 3; ++a) {
-    int v;
-    long long r;
-    launch_choice(c, a, v, r);
-    out[2 * a] = v;
+    const Choice h = launch_choice(c, a);
+    const long long r = h.tile ? c->tile[a].len : h.range;
+    out[2 * a] = h.variant;
     out[2 * a + 1] = (int)(r < 2147483647LL ? r : 2147483647LL);
   }
   return SHASTA_OK;

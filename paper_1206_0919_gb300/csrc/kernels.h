@@ -6,6 +6,7 @@
 #include <stdint.h>
 
 #include "sweep.cuh"
+#include "tile_plan.h"
 
 namespace shasta {
 
@@ -42,6 +43,26 @@ cudaError_t prepare_fuse2();
 cudaError_t launch_fuse2(const SweepParams& P, int nx, int ny, int nz, int axis_a, int axis_b,
                          int eos, int sm_count, cudaStream_t s);
 int sweep_warps_per_block_mixed64();
+// Tiled FP32 / MIXED sweeps (tile_*.cu): bitwise the streaming ones, for the
+// sizes where those are bound by their serial chain.  prepare_* sets the
+// shared-memory attribute of one (axis, shape) kernel and reports its resident
+// blocks per SM (before the first launch or capture).
+cudaError_t prepare_tile_f32_ideal(int axis, int shape, int* blocks_per_sm);
+cudaError_t prepare_tile_f32_bag(int axis, int shape, int* blocks_per_sm);
+cudaError_t prepare_tile_f32_table(int axis, int shape, int* blocks_per_sm);
+cudaError_t prepare_tile_mixed_ideal(int axis, int shape, int* blocks_per_sm);
+cudaError_t prepare_tile_mixed_bag(int axis, int shape, int* blocks_per_sm);
+cudaError_t prepare_tile_mixed64_ideal(int axis, int shape, int* blocks_per_sm);
+cudaError_t prepare_tile_mixed64_bag(int axis, int shape, int* blocks_per_sm);
+cudaError_t launch_tile_f32_ideal(const SweepParams& P, const TilePlan& t, int axis, int sm_count, cudaStream_t s);
+cudaError_t launch_tile_f32_bag(const SweepParams& P, const TilePlan& t, int axis, int sm_count, cudaStream_t s);
+cudaError_t launch_tile_f32_table(const SweepParams& P, const TilePlan& t, int axis, int sm_count, cudaStream_t s);
+cudaError_t launch_tile_mixed_ideal(const SweepParams& P, const TilePlan& t, int axis, int sm_count, cudaStream_t s);
+cudaError_t launch_tile_mixed_bag(const SweepParams& P, const TilePlan& t, int axis, int sm_count, cudaStream_t s);
+cudaError_t launch_tile_mixed64_ideal(const SweepParams& P, const TilePlan& t, int axis, int sm_count,
+                                      cudaStream_t s);
+cudaError_t launch_tile_mixed64_bag(const SweepParams& P, const TilePlan& t, int axis, int sm_count,
+                                    cudaStream_t s);
 // Batched FP32 / MIXED sweeps (one launch over the work list L, all along
 // `axis`); prepare_* as above for the batched kernels.
 cudaError_t prepare_batch_f32(int occupancy[3][3][2]);

@@ -1,0 +1,14 @@
+// tile_mixed64_bag.cu -- tiled sweeps: precision mixed64, bag equation of state.
+#include "sweep_tile_launch.cuh"
+
+namespace shasta {
+
+cudaError_t prepare_tile_mixed64_bag(int axis, int shape, int* blocks_per_sm) {
+  return tile::prepare<EOS_BAG, fast::REC_F64>(axis, shape, blocks_per_sm);
+}
+
+cudaError_t launch_tile_mixed64_bag(const SweepParams& P, const TilePlan& t, int axis, int sm_count, cudaStream_t s) {
+  return tile::launch<EOS_BAG, fast::REC_F64>(P, t, axis, sm_count, s);
+}
+
+}  // namespace shasta
