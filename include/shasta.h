@@ -205,8 +205,10 @@ shasta_status shasta_sweep(shasta_ctx* ctx, int axis);
  * halo per line it touches and about 11 per line end, unless the environment
  * sets SHASTA_BALANCE=0), and the share of work of the CTAs resident on one
  * SM by launch order (1 + s for the first, 1 - s for the last, s timed among
- * 0, 0.04 and 0.08 unless SHASTA_RANK_SKEW sets it).  FP64: the length of the
- * line segments streamed one per thread.  No choice changes results.
+ * 0, 0.04 and 0.08 unless SHASTA_RANK_SKEW sets it).  FP64: nothing where a
+ * block holds whole lines (up to 874 cells; SHASTA_LINES=off in the
+ * environment leaves that out, a number sets the lines per block), else the
+ * length of the line segments streamed one per thread.  No choice changes results.
  * Runs sweeps from the current state into the spare buffer only, so the
  * state is unchanged; synchronous.  Errors: EINVAL (state not set), ECUDA. */
 shasta_status shasta_autotune(shasta_ctx* ctx);

@@ -84,7 +84,8 @@ struct shasta_ctx {
   // FP32 / MIXED: the tiled sweep of each axis (shape -1: none), and the
   // environment's say (shape, or streaming only)
   TilePlan tile[3] = {{-1, 0, 0, 0}, {-1, 0, 0, 0}, {-1, 0, 0, 0}};
-  int force_tile = -1;
+  LinesPlan lines[3] = {};  // FP64: whole-line sweep of each axis (B 0: none)
+  int force_tile = -1, force_lines = 0;
   bool stream_only = false;
   bool tuned = false;     // autotuned launch choice below is valid
   bool tune_tile[3] = {false, false, false};
@@ -401,6 +402,7 @@ constexpr long long kTileAlways = 40, kTileShare = 64;
 Choice launch_choice(const shasta_ctx* c, int axis) {
   Choice h{false, 0, 0};
   if (c->o.precision == SHASTA_FP64) {
+    h.tile = c->lines[axis].B > 0;
     h.range = c->tuned && c->tune_range[axis] > 0 ? c->tune_range[axis] : fp64_segment(c, axis);
     if (c->force_range > 0) h.range = c->force_range;
     return h;
@@ -430,6 +432,7 @@ shasta_status prepare_ranges(shasta_ctx* c) {
 }
 
 cudaError_t launch_tile(shasta_ctx* c, int axis, const SweepParams& P) {
+  if (c->o.precision == SHASTA_FP64) return launch_lines_f64(P, c->lines[axis], axis, c->eos.kind, c->stream);
   const TilePlan& t = c->tile[axis];
   const bool bag = c->eos.kind == SHASTA_EOS_BAG;
   if (c->o.precision == SHASTA_MIXED)
@@ -440,12 +443,24 @@ cudaError_t launch_tile(shasta_ctx* c, int axis, const SweepParams& P) {
   return (bag ? launch_tile_f32_bag : launch_tile_f32_ideal)(P, t, axis, c->sm_count, c->stream);
 }
 
-// Cuts the lines of an axis into tiles and readies the kernel; leaves the
+// Cuts the lines of an axis into tiles (FP64: into blocks of whole lines) and
+// readies the kernel; leaves the
 // axis to the streaming sweep where there is no tiled one.
 cudaError_t plan_tiles(shasta_ctx* c, int axis) {
   TilePlan& t = c->tile[axis];
   t.shape = -1;
   const long long n = axis == 0 ? c->g.nx : (axis == 1 ? c->g.ny : c->g.nz);
+  if (c->o.precision == SHASTA_FP64) {
+    // whole lines wherever one fits a block (up to 874 cells); the reads of
+    // mirrored ghosts want lines of at least the ghost depth
+    LinesPlan& L = c->lines[axis];
+    const long long plane = (long long)c->ncell / n;
+    if (c->stream_only || n < NG || n > 4096 || plane >= (1LL << 31)) return cudaSuccess;
+    const int B = c->force_lines > 0 ? c->force_lines : lines_per_block(plane, (int)n, c->sm_count);
+    if (B < 1 || lines_smem((int)n, B) > kLinesSmem) return cudaSuccess;
+    L = lines_plan_for((int)n, B);
+    return prepare_lines_f64(axis, c->eos.kind, L);
+  }
   if (c->stream_only || n > kTileMaxLine || (long long)c->ncell / n >= (1LL << 31)) return cudaSuccess;
   if (c->o.scheme == SHASTA_SCHEME_SPLIT) return cudaSuccess;
   if (c->o.scheme == SHASTA_SCHEME_NO_ANTIFLUX && c->o.precision == SHASTA_FP32) return cudaSuccess;
@@ -530,8 +545,8 @@ cudaError_t time_choice(shasta_ctx* c, int axis, bool tile, SweepParams P, int w
 // keeps the fastest.  FP32 / MIXED: tiles (alone, untimed, where a warp's
 // streamed share is under kTileAlways), or the register variant and ranges of
 // one line group (no line is cut) or of 1/4 .. 3 ranges per resident warp.
-// FP64: the line segment length (the default one, 24 .. 128 cells, whole
-// lines).  The choice does not change results.
+// FP64: nothing to time on whole lines in shared memory; else the line segment
+// length (the default one, 24 .. 128 cells, whole lines).  The choice does not change results.
 shasta_status autotune(shasta_ctx* c) {
   if (c->o.scheme == SHASTA_SCHEME_SPLIT) {
     c->tuned = true;
@@ -551,6 +566,7 @@ shasta_status autotune(shasta_ctx* c) {
     int bv = 0;
     long long br = f64 ? fp64_segment(c, axis) : n;
     bool bt = false;
+    if (f64 && c->lines[axis].B > 0) continue;
     if (c->tile[axis].shape >= 0) {
       if (c->force_tile >= 0 || stream_share(c, axis) < kTileAlways) {
         c->tune_tile[axis] = true;
@@ -796,6 +812,11 @@ shasta_status shasta_create(const shasta_grid* g, double dx, double lambda, cons
       c->stream_only = true;
     else if (v && *v >= '0' && *v <= '9' && atoi(v) < kTileShapeCount)
       c->force_tile = atoi(v);
+    v = getenv("SHASTA_LINES");
+    if (v && !strcmp(v, "off") && c->o.precision == SHASTA_FP64)
+      c->stream_only = true;
+    else if (v && atoi(v) >= 1 && atoi(v) <= 64)
+      c->force_lines = atoi(v);
   }
   auto bail = [&](cudaError_t err, const char* where) {
     std::string m = std::string(where) + ": " + cudaGetErrorString(err);
@@ -884,10 +905,10 @@ shasta_status shasta_create(const shasta_grid* g, double dx, double lambda, cons
     c->wpb = opts.precision == SHASTA_MIXED        ? sweep_warps_per_block_mixed()
              : opts.precision == SHASTA_MIXED_FP64 ? sweep_warps_per_block_mixed64()
                                                    : sweep_warps_per_block_f32();
-    for (int a = 0; a < 3; ++a) {
-      err = plan_tiles(c, a);
-      if (err != cudaSuccess) return bail(err, "prepare tiled sweep kernels");
-    }
+  }
+  for (int a = 0; a < 3; ++a) {
+    err = plan_tiles(c, a);
+    if (err != cudaSuccess) return bail(err, "prepare tiled sweep kernels");
   }
   if (opts.stream) {
     c->stream = (cudaStream_t)opts.stream;
@@ -1016,7 +1037,8 @@ shasta_status shasta_get_tuning(const shasta_ctx* c, int out[6]) {
   if (!c || !out) return SHASTA_EINVAL;
   for (int a = 0; a < 3; ++a) {
     const Choice h = launch_choice(c, a);
-    const long long r = h.tile ? c->tile[a].len : h.range;
+    const long long n = a == 0 ? c->g.nx : (a == 1 ? c->g.ny : c->g.nz);
+    const long long r = !h.tile ? h.range : (c->o.precision == SHASTA_FP64 ? n : c->tile[a].len);
     out[2 * a] = h.variant;
     out[2 * a + 1] = (int)(r < 2147483647LL ? r : 2147483647LL);
   }

@@ -5,6 +5,7 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include "lines_plan.h"
 #include "sweep.cuh"
 #include "tile_plan.h"
 
@@ -13,6 +14,10 @@ namespace shasta {
 // Fused sweep launchers, one per precision (sweep_f64.cu, sweep_f32.cu,
 // sweep_mixed.cu, sweep_mixed64.cu).  Return the launch error.
 cudaError_t launch_sweep_f64(const SweepParams& P, int axis, int eos, cudaStream_t s);
+// FP64 sweeps on whole lines in shared memory (bitwise the streaming ones);
+// prepare_lines_f64 before the first launch or capture.
+cudaError_t prepare_lines_f64(int axis, int eos, const LinesPlan& t);
+cudaError_t launch_lines_f64(const SweepParams& P, const LinesPlan& t, int axis, int eos, cudaStream_t s);
 cudaError_t launch_sweep_f32(const SweepParams& P, int axis, int eos, cudaStream_t s);
 cudaError_t launch_sweep_mixed(const SweepParams& P, int axis, int eos, cudaStream_t s);
 cudaError_t launch_sweep_mixed64(const SweepParams& P, int axis, int eos, cudaStream_t s);

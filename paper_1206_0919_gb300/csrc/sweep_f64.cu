@@ -2,6 +2,9 @@
 // -fmad=false and IEEE division / square root so that the arithmetic is the
 // plain double-precision evaluation of each expression in source order.
 #include "kernels.h"
+#include "sweep_lines64.cuh"
+
+#include <math.h>
 
 namespace shasta {
 
@@ -13,6 +16,40 @@ static cudaError_t go(const SweepParams& P, cudaStream_t s) {
   long long blocks = (work + threads - 1) / threads;
   sweep_kernel<double, double, EOS, AXIS, false><<<(unsigned)blocks, threads, 0, s>>>(P);
   return cudaGetLastError();
+}
+
+template <int EOS>
+static const void* lines_kernel(int axis) {
+  return axis == 0   ? (const void*)lines64::sweep_lines_kernel<EOS, 0>
+         : axis == 1 ? (const void*)lines64::sweep_lines_kernel<EOS, 1>
+                     : (const void*)lines64::sweep_lines_kernel<EOS, 2>;
+}
+
+static const void* lines_kernel_of(int eos, int axis) {
+  return eos == EOS_IDEAL ? lines_kernel<EOS_IDEAL>(axis)
+                          : (eos == EOS_BAG ? lines_kernel<EOS_BAG>(axis) : lines_kernel<EOS_TABLE>(axis));
+}
+
+cudaError_t prepare_lines_f64(int axis, int eos, const LinesPlan& t) {
+  return cudaFuncSetAttribute(lines_kernel_of(eos, axis), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)kLinesSmem);
+}
+
+cudaError_t launch_lines_f64(const SweepParams& P, const LinesPlan& t, int axis, int eos, cudaStream_t s) {
+  if (P.plane <= 0) return cudaSuccess;
+  if (t.B < 1 || P.n < NG) return cudaErrorInvalidValue;
+  const int np = P.n + 2 * NG;
+  lines64::LineArgs A;
+  A.B = t.B;
+  A.js = axis == 0 ? 1 : t.B;
+  A.ls = axis == 0 ? np : 1;
+  A.sz = t.B * np;
+  A.eta_exp = 0;
+  int ex;
+  if (frexp(P.eta, &ex) == 0.5 && ex <= 0 && ex > -60) A.eta_exp = 1 - ex;
+  void* args[] = {const_cast<SweepParams*>(&P), &A};
+  return cudaLaunchKernel(lines_kernel_of(eos, axis), dim3((unsigned)((P.plane + t.B - 1) / t.B)),
+                          dim3(t.threads), args, t.smem, s);
 }
 
 cudaError_t launch_sweep_f64(const SweepParams& P, int axis, int eos, cudaStream_t s) {
