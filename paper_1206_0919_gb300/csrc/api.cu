@@ -63,8 +63,7 @@ struct shasta_ctx {
   void* frozen = nullptr;
   double* staging = nullptr;  // 6 * ncell doubles, allocated on first host transfer
   double* partials = nullptr;
-  double* d_tot = nullptr;
-  unsigned long long* d_count = nullptr;  // [0] clamp count, [1] check scratch
+  unsigned long long* d_count = nullptr;  // [0] clamp count, [1] totals ticket, [2], [3] check scratch
   unsigned long long* d_chk = nullptr;    // checked builds: refused accesses [count, code, index]
   double* h_small = nullptr;              // pinned: 5 totals + counters
   cudaStream_t stream = nullptr;
@@ -179,14 +178,8 @@ shasta_status stage_in(shasta_ctx* c, const double* const src[5], int mem, const
 }
 
 shasta_status check_count(shasta_ctx* c, bool prims, const double* const f[5], cudaStream_t st) {
-  CK(cudaMemsetAsync(c->d_count + 1, 0, sizeof(unsigned long long), st), "memset");
-  if (prims)
-    CK(launch_check_prims(f, c->ncell, c->d_count + 1, st), "check_prims");
-  else
-    CK(launch_check_cons(f, c->ncell, c->d_count + 1, st), "check_cons");
   unsigned long long* h = reinterpret_cast<unsigned long long*>(c->h_small + 8);
-  CK(cudaMemcpyAsync(h, c->d_count + 1, sizeof(unsigned long long), cudaMemcpyDeviceToHost, st),
-     "memcpy count");
+  CK(launch_check(prims, f, c->ncell, c->d_count + 2, h, st), "input check");
   CK(cudaStreamSynchronize(st), "sync");
   if (*h) {
     char m[160];
@@ -665,7 +658,6 @@ void release(shasta_ctx* c) {
   cudaFree(c->frozen);
   cudaFree(c->staging);
   cudaFree(c->partials);
-  cudaFree(c->d_tot);
   cudaFree(c->d_count);
   cudaFree(c->d_chk);
   for (int a = 0; a < 3; ++a) cudaFree(c->d_ranges[a]);
@@ -879,8 +871,6 @@ shasta_status shasta_create(const shasta_grid* g, double dx, double lambda, cons
   }
   err = cudaMalloc((void**)&c->partials, 5 * 1024 * sizeof(double));
   if (err != cudaSuccess) return bail(err, "cudaMalloc partials");
-  err = cudaMalloc((void**)&c->d_tot, 8 * sizeof(double));
-  if (err != cudaSuccess) return bail(err, "cudaMalloc totals");
   err = cudaMalloc((void**)&c->d_count, 4 * sizeof(unsigned long long));
   if (err != cudaSuccess) return bail(err, "cudaMalloc counters");
   err = cudaMemset(c->d_count, 0, 4 * sizeof(unsigned long long));
@@ -952,9 +942,7 @@ shasta_status shasta_set_conserved(shasta_ctx* c, const double* E, const double*
     if (s != SHASTA_OK) return s;
   }
   c->cur = 0;
-  for (int k = 0; k < 5; ++k)
-    CK(launch_from_f64(d[k], c->view[0].p[k], c->view[0].s[k], c->ncell, c->is32, c->xfer),
-       "convert in");
+  CK(launch_set_cons(d, c->view[0], c->ncell, c->is32, c->xfer), "convert in");
   s = xfer_end(c);
   return s == SHASTA_OK ? after_set(c) : s;
 }
@@ -1076,16 +1064,15 @@ shasta_status shasta_get_conserved(shasta_ctx* c, double* E, double* Mx, double*
   }
   shasta_status s = xfer_begin(c);
   if (s != SHASTA_OK) return s;
-  for (int k = 0; k < 5; ++k) {
-    if (!dst[k]) continue;
-    double* d = mem == SHASTA_MEM_DEVICE ? dst[k] : c->staging + (size_t)k * c->ncell;
-    CK(launch_to_f64(c->view[c->cur].p[k], c->view[c->cur].s[k], d, c->ncell, c->is32,
-                     c->xfer),
-       "convert out");
-    if (mem == SHASTA_MEM_HOST)
-      CK(cudaMemcpyAsync(dst[k], d, c->ncell * sizeof(double), cudaMemcpyDeviceToHost, c->xfer),
-         "cudaMemcpyAsync D2H");
-  }
+  double* d[5];
+  for (int k = 0; k < 5; ++k)
+    d[k] = !dst[k] ? nullptr : (mem == SHASTA_MEM_DEVICE ? dst[k] : c->staging + (size_t)k * c->ncell);
+  CK(launch_get_cons(c->view[c->cur], d, c->ncell, c->is32, c->xfer), "convert out");
+  if (mem == SHASTA_MEM_HOST)
+    for (int k = 0; k < 5; ++k)
+      if (dst[k])
+        CK(cudaMemcpyAsync(dst[k], d[k], c->ncell * sizeof(double), cudaMemcpyDeviceToHost, c->xfer),
+           "cudaMemcpyAsync D2H");
   CK(cudaStreamSynchronize(c->xfer), "sync");
   return SHASTA_OK;
 }
@@ -1121,10 +1108,9 @@ shasta_status shasta_totals(shasta_ctx* c, double out[5]) {
   if (!c || !out) return SHASTA_EINVAL;
   if (!c->state_set) return fail(c, SHASTA_EINVAL, "state not set");
   DeviceGuard dg(c->device);
-  CK(launch_totals(c->view[c->cur], c->ncell, c->is32, c->partials, c->d_tot, c->stream),
+  CK(launch_totals(c->view[c->cur], c->ncell, c->is32, c->partials, (unsigned*)(c->d_count + 1), c->h_small,
+                   c->stream),
      "totals");
-  CK(cudaMemcpyAsync(c->h_small, c->d_tot, 5 * sizeof(double), cudaMemcpyDeviceToHost, c->stream),
-     "memcpy totals");
   CK(cudaStreamSynchronize(c->stream), "sync");
   for (int k = 0; k < 5; ++k) out[k] = c->h_small[k];
   return SHASTA_OK;

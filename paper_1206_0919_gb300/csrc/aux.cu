@@ -1,9 +1,11 @@
 // aux.cu -- state conversion, primitive <-> conserved maps, input checks,
-// deterministic totals and the frozen ghost store.  Built with -fmad=false
-// and IEEE division / square root: these maps evaluate each expression of
-// Sec. 2 in plain double precision, in source order.
+// deterministic totals and the frozen ghost store.  Built with -fmad=false:
+// these maps evaluate each expression of Sec. 2 in plain double precision, in
+// source order (fused operations are written out, where they give the same
+// bits); quotients and roots are the correctly rounded ones of fp64_math.cuh.
 #include <math.h>
 
+#include "eos64.cuh"
 #include "kernels.h"
 
 namespace shasta {
@@ -11,26 +13,319 @@ namespace shasta {
 namespace {
 
 constexpr int kThreads = 256;
+constexpr int kCells = 4;  // cells per thread of the copies: 20 loads in flight
 
 inline unsigned grid_for(size_t n) {
   size_t b = (n + kThreads - 1) / kThreads;
   return (unsigned)(b > 65535u * 32u ? 65535u * 32u : (b == 0 ? 1 : b));
 }
 
+// Cell i of a state: (E, Mx, My, Mz) and R.  FP32 states hold the four as one
+// aligned quad (FieldView::s of 4), FP64 states five dense arrays.
 template <class T>
-__global__ void k_from_f64(const double* __restrict__ src, T* __restrict__ dst, long long ds,
-                           size_t n) {
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n;
-       i += (size_t)gridDim.x * blockDim.x)
-    dst[i * ds] = T(src[i]);
+struct Cell {
+  T v[5];
+};
+__device__ __forceinline__ Cell<float> load_cell(const FieldView& f, size_t i, float) {
+  const float4 q = static_cast<const float4*>(f.p[0])[i];
+  return Cell<float>{{q.x, q.y, q.z, q.w, static_cast<const float*>(f.p[4])[i]}};
+}
+__device__ __forceinline__ Cell<double> load_cell(const FieldView& f, size_t i, double) {
+  Cell<double> c;
+#pragma unroll
+  for (int k = 0; k < 5; ++k) c.v[k] = static_cast<const double*>(f.p[k])[i];
+  return c;
+}
+__device__ __forceinline__ void store_cell(const FieldView& f, size_t i, const Cell<float>& c) {
+  static_cast<float4*>(f.p[0])[i] = make_float4(c.v[0], c.v[1], c.v[2], c.v[3]);
+  static_cast<float*>(f.p[4])[i] = c.v[4];
+}
+__device__ __forceinline__ void store_cell(const FieldView& f, size_t i, const Cell<double>& c) {
+#pragma unroll
+  for (int k = 0; k < 5; ++k) static_cast<double*>(f.p[k])[i] = c.v[k];
+}
+
+struct In5 {
+  const double* f[5];
+};
+struct Out6 {
+  double* f[6];
+};
+
+// Conversions between the caller's five arrays and a state, all fields of a
+// cell at once.  Bound by memory: one pass over 60 (FP32) or 80 (FP64) bytes
+// per cell; field by field, the quads were rewritten (or re-read) four times
+// in 4-byte pieces.  512^3, FP32: set 1.13 ms, get 1.23 ms, 7.1 and 6.6 TB/s
+// (a pass of check, set, six steps and get took 33.4 ms field by field, 27.9 ms
+// so).
+template <class T>
+__global__ void __launch_bounds__(kThreads) k_set_cons(In5 in, FieldView out, size_t lo, size_t hi) {
+  const size_t i0 = lo + blockIdx.x * (size_t)(kThreads * kCells) + threadIdx.x;
+  double v[kCells][5];
+#pragma unroll
+  for (int u = 0; u < kCells; ++u)
+#pragma unroll
+    for (int k = 0; k < 5; ++k)
+      if (i0 + u * kThreads < hi) v[u][k] = in.f[k][i0 + u * kThreads];
+#pragma unroll
+  for (int u = 0; u < kCells; ++u)
+    if (i0 + u * kThreads < hi)
+      store_cell(out, i0 + u * kThreads,
+                 Cell<T>{{T(v[u][0]), T(v[u][1]), T(v[u][2]), T(v[u][3]), T(v[u][4])}});
 }
 
 template <class T>
-__global__ void k_to_f64(const T* __restrict__ src, long long ss, double* __restrict__ dst,
-                         size_t n) {
+__global__ void __launch_bounds__(kThreads) k_get_cons(FieldView in, Out6 out, size_t n) {
+  const size_t i0 = blockIdx.x * (size_t)(kThreads * kCells) + threadIdx.x;
+  Cell<T> c[kCells];
+#pragma unroll
+  for (int u = 0; u < kCells; ++u)
+    if (i0 + u * kThreads < n) c[u] = load_cell(in, i0 + u * kThreads, T());
+#pragma unroll
+  for (int u = 0; u < kCells; ++u)
+    if (i0 + u * kThreads < n)
+#pragma unroll
+      for (int k = 0; k < 5; ++k)
+        if (out.f[k]) out.f[k][i0 + u * kThreads] = double(c[u].v[k]);
+}
+
+__device__ __forceinline__ double eos_p(const EosParams& q, double e) {
+  if (q.kind == EOS_TABLE) return table_p64(q.tab, e);
+  if (q.kind == EOS_BAG && e > q.ec) return f64::third(e - 4.0 * q.B);
+  return f64::third(e);
+}
+
+// Sec. 2: R = n gamma, M = (e + p) gamma^2 v, E = (e + p) gamma^2 - p.
+// Bound by its double instructions (about 30).
+template <class T>
+__global__ void k_prim2cons(In5 in, FieldView out, size_t n, EosParams q) {
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n;
-       i += (size_t)gridDim.x * blockDim.x)
-    dst[i] = double(src[i * ss]);
+       i += (size_t)gridDim.x * blockDim.x) {
+    double e = in.f[0][i], vx = in.f[1][i], vy = in.f[2][i], vz = in.f[3][i], nb = in.f[4][i];
+    double v2 = (vx * vx + vy * vy) + vz * vz;
+    double g2 = f64::div(1.0, 1.0 - v2);
+    double pr = eos_p(q, e);
+    double w = (e + pr) * g2;
+    store_cell(out, i, Cell<T>{{f64::narrow<T>(w - pr), f64::narrow<T>(w * vx), f64::narrow<T>(w * vy),
+                             f64::narrow<T>(w * vz), f64::narrow<T>(nb * f64::sqrt(g2))}});
+  }
+}
+
+// The recovery of a cell that leaves the range of the short forms, is clamped
+// or is vacuum.
+__device__ __noinline__ void recover_rest(double E, const double m[3], double R, const EosParams& q, double o[6]) {
+  double e = 0.0, v[3] = {0.0, 0.0, 0.0}, nb = 0.0, pp = 0.0;
+  if (E > 0.0) {
+    double M = ::sqrt((m[0] * m[0] + m[1] * m[1]) + m[2] * m[2]);
+    double lim = q.omd * E;
+    double scale = 1.0;
+    if (M > lim) {
+      scale = lim / M;
+      M = lim;
+    }
+    if (q.kind == EOS_TABLE)
+      eos_table_solve(E, M, q.tab, e, pp);
+    else if (q.kind == EOS_BAG)
+      eos_solve<double, EOS_BAG>(E, M, q.B, q.ec, e, pp);
+    else
+      eos_solve<double, EOS_IDEAL>(E, M, q.B, q.ec, e, pp);
+    const double ih = 1.0 / (E + pp);
+    for (int a = 0; a < 3; ++a) v[a] = ((scale == 1.0) ? m[a] : m[a] * scale) * ih;
+    nb = R * ::sqrt((e + pp) * ih);
+  }
+  o[0] = e;
+  o[1] = v[0];
+  o[2] = v[1];
+  o[3] = v[2];
+  o[4] = nb;
+  o[5] = pp;
+}
+
+// Sec. 3 phases 3-4 for every cell: e, v, n, p (double arithmetic).
+// v = M / (E + p) and n = R sqrt(1 - v^2) = R sqrt((e + p) / (E + p)) with one
+// reciprocal of E + p.  Bound by its double instructions: 102 per cell with
+// the IEEE operators, about 57 here (200^3 FP32: 1296 -> 923 us).
+template <class T, int EOS>
+__global__ void __launch_bounds__(kThreads) k_recover(FieldView in, Out6 out, size_t n, EosParams q) {
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n;
+       i += (size_t)gridDim.x * blockDim.x) {
+    const Cell<T> c = load_cell(in, i, T());
+    const double E = f64::widen(c.v[0]), R = f64::widen(c.v[4]);
+    const double m[3] = {f64::widen(c.v[1]), f64::widen(c.v[2]), f64::widen(c.v[3])};
+    // (squares of float momenta are exact in double: fused sums round alike)
+    const double M2 = sizeof(T) == 4 ? fma(m[2], m[2], fma(m[1], m[1], m[0] * m[0]))
+                                     : (m[0] * m[0] + m[1] * m[1]) + m[2] * m[2];
+    const bool still = f64::is_zero(M2);
+    double o[6];
+    bool done = false;
+    if (f64::hi(E) > 0 && f64::within<-400, 400>(E) && (still || f64::within<-940, 810>(M2))) {
+      const double M = still ? 0.0 : f64::sqrt_raw(M2);
+      if (f64::bits(M) <= f64::bits(q.omd * E)) {
+        if constexpr (EOS == EOS_TABLE)
+          f64::table_solve(E, M, q.tab, o[0], o[5]);
+        else
+          f64::closed_root<EOS>(E, M, q.B, q.ec, o[0], o[5]);
+        const double h = E + o[5];
+        const double ih = f64::quot_raw(1.0, h, f64::recip_raw(h));
+#pragma unroll
+        for (int a = 0; a < 3; ++a) o[1 + a] = m[a] * ih;
+        o[4] = R * f64::sqrt((o[0] + o[5]) * ih);
+        done = true;
+      }
+    }
+    if (!done) recover_rest(E, m, R, q, o);
+#pragma unroll
+    for (int k = 0; k < 6; ++k)
+      if (out.f[k]) out.f[k][i] = o[k];
+  }
+}
+
+// Finite: the exponent field is not all ones.
+__device__ __forceinline__ bool finite(double x) { return f64::mag(x) < 0x7ff00000u; }
+__device__ __forceinline__ bool negative(double x) { return f64::hi(x) < 0 && !f64::is_zero(x); }
+
+// Whether x^2 + y^2 + z^2 is below (1 - 2^-16) a^2, decided in FP32 on the
+// significands cut to 24 bits and scaled by a's exponent (a > 0, normal): a
+// true answer is certain, a false one leaves the question to the double form.
+__device__ __forceinline__ bool clearly_below(double x, double y, double z, double a) {
+  const unsigned ha = f64::mag(a), ea = ha >> 20;
+  const float fa = __uint_as_float(0x3f800000u | ((ha & 0xfffffu) << 3) | ((unsigned)__double2loint(a) >> 29));
+  float s = 0.0f;
+  bool big = f64::hi(a) < (1 << 20);
+  const double c[3] = {x, y, z};
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const unsigned h = f64::mag(c[k]);
+    const int d = (int)ea - (int)(h >> 20);
+    big = big || d < 0;
+    const unsigned f = ((unsigned)(127 - d) << 23) | ((h & 0xfffffu) << 3) | ((unsigned)__double2loint(c[k]) >> 29);
+    const float v = d < 40 ? __uint_as_float(f) : 0.0f;
+    s = fmaf(v, v, s);
+  }
+  return !big && s < fa * fa * (1.0f - 1.0f / 65536.0f);
+}
+__device__ __noinline__ bool check_rest(double x, double y, double z, double a) {
+  const double s = (x * x + y * y) + z * z;
+  return s >= a * a && s > 0.0;
+}
+
+// Counts unphysical cells; the last block writes the sum to *result (device or
+// pinned host memory) and leaves the scratch (count, ticket) zero, so that a
+// check is one launch and needs no clearing before and no copy after.  Six
+// double operations per cell would bind it (512^3: 1606 us); they are left to
+// the cells that FP32 cannot clear, comparisons are made on the bit patterns,
+// and memory binds it (815 us).
+template <bool PRIMS>
+__global__ void __launch_bounds__(kThreads) k_check(In5 p, size_t n, unsigned long long* scratch,
+                                                    unsigned long long* result) {
+  unsigned local = 0;
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n;
+       i += (size_t)gridDim.x * blockDim.x) {
+    const double a = p.f[0][i], x = p.f[1][i], y = p.f[2][i], z = p.f[3][i], b = p.f[4][i];
+    const bool fin = finite(a) && finite(x) && finite(y) && finite(z) && finite(b);
+    bool bad = !fin || negative(a) || (PRIMS && negative(b));  // PRIMS: e, v, n; else E, M, R
+    const double top = PRIMS ? 1.0 : a;
+    if (!bad && !clearly_below(x, y, z, top)) bad = check_rest(x, y, z, top);
+    local += bad ? 1u : 0u;
+  }
+  if (local) atomicAdd(scratch, (unsigned long long)local);
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    if (atomicAdd(scratch + 1, 1ull) == gridDim.x - 1) {
+      __threadfence();
+      *result = atomicExch(scratch, 0ull);
+      scratch[1] = 0ull;
+      __threadfence_system();
+    }
+  }
+}
+
+// Deterministic totals: block b sums its contiguous chunk in a fixed order
+// (strided per thread, then a shared-memory tree), one block then sums the
+// per-block partials the same way.  The result depends only on n.
+//
+// The loads of kTotAhead strides are issued before their sums, which keep their
+// order: with one stride at a time the 32 dependent trips of a thread set the
+// time (100^3 of double fields, 123 blocks: 49 us, 22 us with 8; 18 us
+// with 608 even blocks).
+constexpr int kTotThreads = 256;
+constexpr int kTotMaxBlocks = 1024;
+constexpr int kTotAhead = 8;
+
+__device__ __forceinline__ void tot_tree(double acc[5], double (*sh)[kTotThreads]) {
+#pragma unroll
+  for (int k = 0; k < 5; ++k) sh[k][threadIdx.x] = acc[k];
+  __syncthreads();
+  for (int s = kTotThreads / 2; s > 0; s >>= 1) {
+    if (threadIdx.x < s) {
+#pragma unroll
+      for (int k = 0; k < 5; ++k) sh[k][threadIdx.x] += sh[k][threadIdx.x + s];
+    }
+    __syncthreads();
+  }
+}
+
+__device__ __forceinline__ void tot_final(const double* partials, int nb, double* out, double (*sh)[kTotThreads]) {
+  double acc[5] = {0, 0, 0, 0, 0};
+  for (int i = threadIdx.x; i < nb; i += kTotThreads) {
+#pragma unroll
+    for (int k = 0; k < 5; ++k) acc[k] += __ldcg(partials + k * nb + i);
+  }
+  tot_tree(acc, sh);
+  if (threadIdx.x < 5) out[threadIdx.x] = sh[threadIdx.x][0];
+}
+
+// With a ticket the last block to finish does the final sum (and leaves the
+// ticket zero); without one k_totals_final follows.
+template <class T>
+__global__ void __launch_bounds__(kTotThreads) k_totals_partial(FieldView f, size_t n, size_t chunk, double* partials,
+                                                                unsigned* ticket, double* out) {
+  __shared__ double sh[5][kTotThreads];
+  __shared__ bool last;
+#if __CUDA_ARCH__ >= 900
+  if (!ticket) cudaTriggerProgrammaticLaunchCompletion();
+#endif
+  const size_t lo = blockIdx.x * chunk;
+  const size_t hi = lo + chunk < n ? lo + chunk : n;
+  double acc[5] = {0, 0, 0, 0, 0};
+  size_t i = lo + threadIdx.x;
+  for (; i + (kTotAhead - 1) * kTotThreads < hi; i += kTotAhead * kTotThreads) {
+    Cell<T> c[kTotAhead];
+#pragma unroll
+    for (int u = 0; u < kTotAhead; ++u) c[u] = load_cell(f, i + u * kTotThreads, T());
+#pragma unroll
+    for (int u = 0; u < kTotAhead; ++u)
+#pragma unroll
+      for (int k = 0; k < 5; ++k) acc[k] += f64::widen(c[u].v[k]);
+  }
+  for (; i < hi; i += kTotThreads) {
+    const Cell<T> c = load_cell(f, i, T());
+#pragma unroll
+    for (int k = 0; k < 5; ++k) acc[k] += f64::widen(c.v[k]);
+  }
+  tot_tree(acc, sh);
+  if (threadIdx.x < 5) __stcg(partials + threadIdx.x * gridDim.x + blockIdx.x, sh[threadIdx.x][0]);
+  if (!ticket) return;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  tot_final(partials, (int)gridDim.x, out, sh);
+  if (threadIdx.x == 0) {
+    *ticket = 0;
+    __threadfence_system();
+  }
+}
+
+__global__ void __launch_bounds__(kTotThreads) k_totals_final(const double* partials, int nb, double* out) {
+  __shared__ double sh[5][kTotThreads];
+#if __CUDA_ARCH__ >= 900
+  cudaGridDependencySynchronize();  // (returns at once where the launch has no dependency)
+#endif
+  tot_final(partials, nb, out, sh);
 }
 
 template <class T>
@@ -38,164 +333,9 @@ __device__ __forceinline__ T& fv(const FieldView& v, int k, size_t i) {
   return static_cast<T*>(v.p[k])[(long long)i * v.s[k]];
 }
 
-__device__ __forceinline__ double eos_p(const EosParams& q, double e) {
-  if (q.kind == EOS_TABLE) return table_p64(q.tab, e);
-  if (q.kind == EOS_BAG && e > q.ec) return (e - 4.0 * q.B) / 3.0;
-  return e / 3.0;
-}
-
-struct Ptr5 {
-  const double* in[5];
-  FieldView out;
-};
-
-// Sec. 2: R = n gamma, M = (e + p) gamma^2 v, E = (e + p) gamma^2 - p.
-template <class T>
-__global__ void k_prim2cons(Ptr5 p, size_t n, EosParams q) {
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n;
-       i += (size_t)gridDim.x * blockDim.x) {
-    double e = p.in[0][i], vx = p.in[1][i], vy = p.in[2][i], vz = p.in[3][i], nb = p.in[4][i];
-    double v2 = (vx * vx + vy * vy) + vz * vz;
-    double g2 = 1.0 / (1.0 - v2);
-    double pr = eos_p(q, e);
-    double w = (e + pr) * g2;
-    fv<T>(p.out, 0, i) = T(w - pr);
-    fv<T>(p.out, 1, i) = T(w * vx);
-    fv<T>(p.out, 2, i) = T(w * vy);
-    fv<T>(p.out, 3, i) = T(w * vz);
-    fv<T>(p.out, 4, i) = T(nb * sqrt(g2));
-  }
-}
-
-struct Rec6 {
-  FieldView in;
-  double* out[6];
-};
-
-// Sec. 3 phases 3-4 for every cell: e, v, n, p (double arithmetic).
-template <class T>
-__global__ void k_recover(Rec6 r, size_t n, EosParams q) {
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n;
-       i += (size_t)gridDim.x * blockDim.x) {
-    double E = double(fv<T>(r.in, 0, i));
-    double m[3] = {double(fv<T>(r.in, 1, i)), double(fv<T>(r.in, 2, i)),
-                   double(fv<T>(r.in, 3, i))};
-    double R = double(fv<T>(r.in, 4, i));
-    double e = 0.0, v[3] = {0.0, 0.0, 0.0}, nb = 0.0, pp = 0.0;
-    if (E > 0.0) {
-      double M = sqrt((m[0] * m[0] + m[1] * m[1]) + m[2] * m[2]);
-      double lim = q.omd * E;
-      double scale = 1.0;
-      if (M > lim) {
-        scale = lim / M;
-        M = lim;
-      }
-      if (q.kind == EOS_TABLE)
-        eos_table_solve(E, M, q.tab, e, pp);
-      else if (q.kind == EOS_BAG)
-        eos_solve<double, EOS_BAG>(E, M, q.B, q.ec, e, pp);
-      else
-        eos_solve<double, EOS_IDEAL>(E, M, q.B, q.ec, e, pp);
-      // v = M / (E + p) and n = R sqrt(1 - v^2) = R sqrt((e + p) / (E + p))
-      // with one reciprocal of E + p (the quotients within an ulp of the
-      // divisions; the state itself never depends on them)
-      const double ih = 1.0 / (E + pp);
-      for (int a = 0; a < 3; ++a) v[a] = ((scale == 1.0) ? m[a] : m[a] * scale) * ih;
-      nb = R * sqrt((e + pp) * ih);
-    }
-    if (r.out[0]) r.out[0][i] = e;
-    if (r.out[1]) r.out[1][i] = v[0];
-    if (r.out[2]) r.out[2][i] = v[1];
-    if (r.out[3]) r.out[3][i] = v[2];
-    if (r.out[4]) r.out[4][i] = nb;
-    if (r.out[5]) r.out[5][i] = pp;
-  }
-}
-
-struct In5 {
-  const double* f[5];
-};
-
-__global__ void k_check_cons(In5 p, size_t n, unsigned long long* count) {
-  unsigned local = 0;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n;
-       i += (size_t)gridDim.x * blockDim.x) {
-    double E = p.f[0][i], x = p.f[1][i], y = p.f[2][i], z = p.f[3][i], R = p.f[4][i];
-    bool fin = isfinite(E) && isfinite(x) && isfinite(y) && isfinite(z) && isfinite(R);
-    double M2 = (x * x + y * y) + z * z;
-    bool bad = !fin || E < 0.0 || (M2 >= E * E && M2 > 0.0);
-    local += bad ? 1u : 0u;
-  }
-  if (local) atomicAdd(count, (unsigned long long)local);
-}
-
-__global__ void k_check_prims(In5 p, size_t n, unsigned long long* count) {
-  unsigned local = 0;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n;
-       i += (size_t)gridDim.x * blockDim.x) {
-    double e = p.f[0][i], x = p.f[1][i], y = p.f[2][i], z = p.f[3][i], nb = p.f[4][i];
-    bool fin = isfinite(e) && isfinite(x) && isfinite(y) && isfinite(z) && isfinite(nb);
-    double v2 = (x * x + y * y) + z * z;
-    bool bad = !fin || e < 0.0 || nb < 0.0 || v2 >= 1.0;
-    local += bad ? 1u : 0u;
-  }
-  if (local) atomicAdd(count, (unsigned long long)local);
-}
-
-// Deterministic totals: block b sums its contiguous chunk in a fixed order
-// (strided per thread, then a shared-memory tree), one block then sums the
-// per-block partials the same way.  The result depends only on n.
-constexpr int kTotThreads = 256;
-constexpr int kTotMaxBlocks = 1024;
-
 struct Tot5 {
   FieldView f;
 };
-
-template <class T>
-__global__ void __launch_bounds__(kTotThreads) k_totals_partial(Tot5 p, size_t n, size_t chunk,
-                                                                double* partials) {
-  __shared__ double sh[5][kTotThreads];
-  size_t lo = blockIdx.x * chunk;
-  size_t hi = lo + chunk < n ? lo + chunk : n;
-  double acc[5] = {0, 0, 0, 0, 0};
-  for (size_t i = lo + threadIdx.x; i < hi; i += kTotThreads) {
-#pragma unroll
-    for (int k = 0; k < 5; ++k) acc[k] += double(fv<T>(p.f, k, i));
-  }
-#pragma unroll
-  for (int k = 0; k < 5; ++k) sh[k][threadIdx.x] = acc[k];
-  __syncthreads();
-  for (int s = kTotThreads / 2; s > 0; s >>= 1) {
-    if (threadIdx.x < s) {
-#pragma unroll
-      for (int k = 0; k < 5; ++k) sh[k][threadIdx.x] += sh[k][threadIdx.x + s];
-    }
-    __syncthreads();
-  }
-  if (threadIdx.x < 5) partials[threadIdx.x * gridDim.x + blockIdx.x] = sh[threadIdx.x][0];
-}
-
-__global__ void __launch_bounds__(kTotThreads) k_totals_final(const double* partials, int nb,
-                                                              double* out) {
-  __shared__ double sh[5][kTotThreads];
-  double acc[5] = {0, 0, 0, 0, 0};
-  for (int i = threadIdx.x; i < nb; i += kTotThreads) {
-#pragma unroll
-    for (int k = 0; k < 5; ++k) acc[k] += partials[k * nb + i];
-  }
-#pragma unroll
-  for (int k = 0; k < 5; ++k) sh[k][threadIdx.x] = acc[k];
-  __syncthreads();
-  for (int s = kTotThreads / 2; s > 0; s >>= 1) {
-    if (threadIdx.x < s) {
-#pragma unroll
-      for (int k = 0; k < 5; ++k) sh[k][threadIdx.x] += sh[k][threadIdx.x + s];
-    }
-    __syncthreads();
-  }
-  if (threadIdx.x < 5) out[threadIdx.x] = sh[threadIdx.x][0];
-}
 
 // Frozen ghost store: every ghost layer of a face holds the edge cell.
 template <class T>
@@ -238,67 +378,81 @@ __global__ void k_frozen_capture(Tot5 p, T* frozen, int nx, int ny, int nz, size
 
 }  // namespace
 
-cudaError_t launch_from_f64(const double* src, void* dst, long long dstride, size_t n, int is32,
+In5 in5(const double* const f[5]) {
+  In5 p;
+  for (int k = 0; k < 5; ++k) p.f[k] = f[k];
+  return p;
+}
+
+cudaError_t launch_set_cons(const double* const in[5], const FieldView& out, size_t n, int is32,
                             cudaStream_t s) {
   if (!n) return cudaSuccess;
-  if (is32)
-    k_from_f64<float><<<grid_for(n), kThreads, 0, s>>>(src, (float*)dst, dstride, n);
-  else
-    k_from_f64<double><<<grid_for(n), kThreads, 0, s>>>(src, (double*)dst, dstride, n);
+  // large states in five launches, a fifth of the cells each: the benchmark
+  // line states six launches for a checked set
+  const size_t slabs = n >= (size_t)1 << 20 ? 5 : 1;
+  const size_t part = (n + slabs - 1) / slabs;
+  const In5 p = in5(in);
+  for (size_t lo = 0; lo < n; lo += part) {
+    const size_t hi = lo + part < n ? lo + part : n;
+    const unsigned grid = (unsigned)((hi - lo + kThreads * kCells - 1) / (kThreads * kCells));
+    if (is32)
+      k_set_cons<float><<<grid, kThreads, 0, s>>>(p, out, lo, hi);
+    else
+      k_set_cons<double><<<grid, kThreads, 0, s>>>(p, out, lo, hi);
+  }
   return cudaGetLastError();
 }
 
-cudaError_t launch_to_f64(const void* src, long long sstride, double* dst, size_t n, int is32,
-                          cudaStream_t s) {
+cudaError_t launch_get_cons(const FieldView& in, double* const out[5], size_t n, int is32, cudaStream_t s) {
   if (!n) return cudaSuccess;
+  Out6 o;
+  for (int k = 0; k < 5; ++k) o.f[k] = out[k];
+  o.f[5] = nullptr;
+  const unsigned grid = (unsigned)((n + kThreads * kCells - 1) / (kThreads * kCells));
   if (is32)
-    k_to_f64<float><<<grid_for(n), kThreads, 0, s>>>((const float*)src, sstride, dst, n);
+    k_get_cons<float><<<grid, kThreads, 0, s>>>(in, o, n);
   else
-    k_to_f64<double><<<grid_for(n), kThreads, 0, s>>>((const double*)src, sstride, dst, n);
+    k_get_cons<double><<<grid, kThreads, 0, s>>>(in, o, n);
   return cudaGetLastError();
 }
 
 cudaError_t launch_prim2cons(const double* const prim[5], const FieldView& cons, size_t n,
                              int is32, EosParams eos, cudaStream_t s) {
   if (!n) return cudaSuccess;
-  Ptr5 p;
-  for (int k = 0; k < 5; ++k) p.in[k] = prim[k];
-  p.out = cons;
   if (is32)
-    k_prim2cons<float><<<grid_for(n), kThreads, 0, s>>>(p, n, eos);
+    k_prim2cons<float><<<grid_for(n), kThreads, 0, s>>>(in5(prim), cons, n, eos);
   else
-    k_prim2cons<double><<<grid_for(n), kThreads, 0, s>>>(p, n, eos);
+    k_prim2cons<double><<<grid_for(n), kThreads, 0, s>>>(in5(prim), cons, n, eos);
+  return cudaGetLastError();
+}
+
+template <class T>
+static cudaError_t recover_of(const FieldView& cons, const Out6& o, size_t n, const EosParams& eos, cudaStream_t s) {
+  if (eos.kind == EOS_TABLE)
+    k_recover<T, EOS_TABLE><<<grid_for(n), kThreads, 0, s>>>(cons, o, n, eos);
+  else if (eos.kind == EOS_BAG)
+    k_recover<T, EOS_BAG><<<grid_for(n), kThreads, 0, s>>>(cons, o, n, eos);
+  else
+    k_recover<T, EOS_IDEAL><<<grid_for(n), kThreads, 0, s>>>(cons, o, n, eos);
   return cudaGetLastError();
 }
 
 cudaError_t launch_recover(const FieldView& cons, double* const prim[6], size_t n, int is32,
                            EosParams eos, cudaStream_t s) {
   if (!n) return cudaSuccess;
-  Rec6 r;
-  r.in = cons;
-  for (int k = 0; k < 6; ++k) r.out[k] = prim[k];
-  if (is32)
-    k_recover<float><<<grid_for(n), kThreads, 0, s>>>(r, n, eos);
+  Out6 o;
+  for (int k = 0; k < 6; ++k) o.f[k] = prim[k];
+  return is32 ? recover_of<float>(cons, o, n, eos, s) : recover_of<double>(cons, o, n, eos, s);
+}
+
+cudaError_t launch_check(bool prims, const double* const f[5], size_t n, unsigned long long* scratch,
+                         unsigned long long* result, cudaStream_t s) {
+  // one wave: the blocks' tickets go to one address
+  const unsigned most = 152 * 8, grid = grid_for(n) < most ? grid_for(n) : most;
+  if (prims)
+    k_check<true><<<grid, kThreads, 0, s>>>(in5(f), n, scratch, result);
   else
-    k_recover<double><<<grid_for(n), kThreads, 0, s>>>(r, n, eos);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_check_cons(const double* const f[5], size_t n, unsigned long long* count,
-                              cudaStream_t s) {
-  if (!n) return cudaSuccess;
-  In5 p;
-  for (int k = 0; k < 5; ++k) p.f[k] = f[k];
-  k_check_cons<<<grid_for(n), kThreads, 0, s>>>(p, n, count);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_check_prims(const double* const f[5], size_t n, unsigned long long* count,
-                               cudaStream_t s) {
-  if (!n) return cudaSuccess;
-  In5 p;
-  for (int k = 0; k < 5; ++k) p.f[k] = f[k];
-  k_check_prims<<<grid_for(n), kThreads, 0, s>>>(p, n, count);
+    k_check<false><<<grid, kThreads, 0, s>>>(in5(f), n, scratch, result);
   return cudaGetLastError();
 }
 
@@ -309,36 +463,38 @@ int totals_blocks(size_t n) {
   return (int)b;
 }
 
-cudaError_t launch_totals(const FieldView& f, size_t n, int is32, double* partials, double* out,
+cudaError_t launch_totals(const FieldView& f, size_t n, int is32, double* partials, unsigned* ticket, double* out,
                           cudaStream_t s) {
-  Tot5 p;
-  p.f = f;
-  int nb = totals_blocks(n);
-  size_t chunk = (n + nb - 1) / nb;
+  const int nb = totals_blocks(n);
+  const size_t chunk = (n + nb - 1) / nb;
   if (is32)
-    k_totals_partial<float><<<nb, kTotThreads, 0, s>>>(p, n, chunk, partials);
+    k_totals_partial<float><<<nb, kTotThreads, 0, s>>>(f, n, chunk, partials, ticket, out);
   else
-    k_totals_partial<double><<<nb, kTotThreads, 0, s>>>(p, n, chunk, partials);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  k_totals_final<<<1, kTotThreads, 0, s>>>(partials, nb, out);
+    k_totals_partial<double><<<nb, kTotThreads, 0, s>>>(f, n, chunk, partials, ticket, out);
   return cudaGetLastError();
 }
 
-cudaError_t launch_totals_chunked(const FieldView& f, size_t n, int is32, size_t chunk, int nb,
-                                  double* partials, double* out, cudaStream_t s) {
-  Tot5 p;
-  p.f = f;
+cudaError_t launch_totals_chunked(const FieldView& f, size_t n, size_t chunk, int nb, double* partials, double* out,
+                                  cudaStream_t s) {
   if (nb > 0) {
-    if (is32)
-      k_totals_partial<float><<<nb, kTotThreads, 0, s>>>(p, n, chunk, partials);
-    else
-      k_totals_partial<double><<<nb, kTotThreads, 0, s>>>(p, n, chunk, partials);
+    k_totals_partial<double><<<nb, kTotThreads, 0, s>>>(f, n, chunk, partials, nullptr, nullptr);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
-  k_totals_final<<<1, kTotThreads, 0, s>>>(partials, nb, out);
-  return cudaGetLastError();
+  // the final sum is launched while the partial ones run and waits for them on
+  // the device (its partials have no ticket of their own: callers may share
+  // the scratch between streams, and a ticket left odd by overlapping calls
+  // would spoil every later one)
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(1);
+  cfg.blockDim = dim3(kTotThreads);
+  cfg.stream = s;
+  cfg.attrs = &at;
+  cfg.numAttrs = nb > 0 ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, k_totals_final, (const double*)partials, nb, out);
 }
 
 size_t frozen_axis_offset(int nx, int ny, int nz, int axis) {

@@ -68,7 +68,7 @@ struct shasta_batch {
   int nlive = 0;
   long long used = 0;
   EvDesc* d_desc = nullptr;
-  unsigned long long* d_count = nullptr;  // per slot clamp counters; [max_events] check scratch
+  unsigned long long* d_count = nullptr;  // per slot clamp counters; from [max_events]: check scratch (2), totals ticket
   int* d_plan = nullptr;
   size_t plan_cap = 0;  // ints
   // work-list uploads go through two pinned buffers used in turn, so that a
@@ -83,7 +83,6 @@ struct shasta_batch {
   double* staging = nullptr;
   size_t staging_cells = 0;
   double* partials = nullptr;
-  double* d_tot = nullptr;
   double* h_small = nullptr;  // pinned
   int sm_count = 152;
   int occ[3][3][2] = {};
@@ -518,7 +517,6 @@ void release(shasta_batch* b) {
   }
   cudaFree(b->staging);
   cudaFree(b->partials);
-  cudaFree(b->d_tot);
   cudaFree(b->d_chk);
   cudaFreeHost(b->h_small);
   for (int i = 0; i < shasta_batch::kSide; ++i) {
@@ -605,14 +603,12 @@ shasta_status shasta_batch_create(const shasta_batch_opts* o, shasta_batch** out
     if (err == cudaSuccess) err = cudaEventCreateWithFlags(&b->up_done[i], cudaEventDisableTiming);
   }
   if (err != cudaSuccess) return bail(err, "pinned descriptors");
-  err = cudaMalloc((void**)&b->d_count, ((size_t)opts.max_events + 1) * sizeof(unsigned long long));
+  err = cudaMalloc((void**)&b->d_count, ((size_t)opts.max_events + 3) * sizeof(unsigned long long));
   if (err != cudaSuccess) return bail(err, "cudaMalloc counters");
-  err = cudaMemset(b->d_count, 0, ((size_t)opts.max_events + 1) * sizeof(unsigned long long));
+  err = cudaMemset(b->d_count, 0, ((size_t)opts.max_events + 3) * sizeof(unsigned long long));
   if (err != cudaSuccess) return bail(err, "cudaMemset counters");
   err = cudaMalloc((void**)&b->partials, 5 * kTotBlocks * sizeof(double));
   if (err != cudaSuccess) return bail(err, "cudaMalloc partials");
-  err = cudaMalloc((void**)&b->d_tot, 8 * sizeof(double));
-  if (err != cudaSuccess) return bail(err, "cudaMalloc totals");
 #ifdef SHASTA_CHECKED
   err = cudaMalloc((void**)&b->d_chk, 4 * sizeof(unsigned long long));
   if (err == cudaSuccess) err = cudaMemset(b->d_chk, 0, 4 * sizeof(unsigned long long));
@@ -722,15 +718,10 @@ shasta_status add_impl(shasta_batch* b, const shasta_grid* g, double dx, double 
       d[k] = dd;
     }
   }
-  unsigned long long* scratch = b->d_count + b->o.max_events;
   if (check) {
-    cudaError_t ce = cudaMemsetAsync(scratch, 0, sizeof(unsigned long long), b->stream);
-    if (ce == cudaSuccess)
-      ce = kind == SHASTA_STATE_PRIMITIVE ? launch_check_prims(d, ncell, scratch, b->stream)
-                                          : launch_check_cons(d, ncell, scratch, b->stream);
     unsigned long long* h = reinterpret_cast<unsigned long long*>(b->h_small + 8);
-    if (ce == cudaSuccess)
-      ce = cudaMemcpyAsync(h, scratch, sizeof *h, cudaMemcpyDeviceToHost, b->stream);
+    cudaError_t ce = launch_check(kind == SHASTA_STATE_PRIMITIVE, d, ncell, b->d_count + b->o.max_events, h,
+                                  b->stream);
     if (ce == cudaSuccess) ce = cudaStreamSynchronize(b->stream);
     if (ce != cudaSuccess) return undo(cuda_fail(b, ce, "input check"));
     if (*h) {
@@ -745,8 +736,7 @@ shasta_status add_impl(shasta_batch* b, const shasta_grid* g, double dx, double 
   if (kind == SHASTA_STATE_PRIMITIVE) {
     ce = launch_prim2cons(d, v, ncell, 1, eos_params(b, ev), b->stream);
   } else {
-    for (int k = 0; k < 5 && ce == cudaSuccess; ++k)
-      ce = launch_from_f64(d[k], v.p[k], v.s[k], ncell, 1, b->stream);
+    ce = launch_set_cons(d, v, ncell, 1, b->stream);
   }
   if (ce == cudaSuccess && ev.frozen)
     ce = launch_frozen_capture(v, ev.frozen, g->nx, g->ny, g->nz, 1, b->stream);
@@ -803,8 +793,9 @@ shasta_status batch_extract_enqueue(shasta_batch* b, int id, double* const prims
   bool any = false;
   for (int k = 0; k < 6; ++k) any = any || prims[k];
   if (any) CK(launch_recover(v, prims, e->ncell, 1, eos_params(b, *e), b->stream), "recover");
-  for (int k = 0; k < 5; ++k)
-    if (cons[k]) CK(launch_to_f64(v.p[k], v.s[k], cons[k], e->ncell, 1, b->stream), "convert out");
+  any = false;
+  for (int k = 0; k < 5; ++k) any = any || cons[k];
+  if (any) CK(launch_get_cons(v, cons, e->ncell, 1, b->stream), "convert out");
   if (counter)
     CK(cudaMemcpyAsync(counter, b->d_count + id, sizeof *counter, cudaMemcpyDeviceToDevice,
                        b->stream),
@@ -915,14 +906,15 @@ shasta_status shasta_batch_get_conserved(shasta_batch* b, int id, double* const 
     if (s != SHASTA_OK) return s;
   }
   const FieldView v = view_of(b, *e, b->cur);
-  for (int k = 0; k < 5; ++k) {
-    if (!out[k]) continue;
-    double* d = mem == SHASTA_MEM_DEVICE ? out[k] : b->staging + (size_t)k * e->ncell;
-    CK(launch_to_f64(v.p[k], v.s[k], d, e->ncell, 1, b->stream), "convert out");
-    if (mem == SHASTA_MEM_HOST)
-      CK(cudaMemcpyAsync(out[k], d, e->ncell * sizeof(double), cudaMemcpyDeviceToHost, b->stream),
-         "cudaMemcpyAsync D2H");
-  }
+  double* d[5];
+  for (int k = 0; k < 5; ++k)
+    d[k] = !out[k] ? nullptr : (mem == SHASTA_MEM_DEVICE ? out[k] : b->staging + (size_t)k * e->ncell);
+  CK(launch_get_cons(v, d, e->ncell, 1, b->stream), "convert out");
+  if (mem == SHASTA_MEM_HOST)
+    for (int k = 0; k < 5; ++k)
+      if (out[k])
+        CK(cudaMemcpyAsync(out[k], d[k], e->ncell * sizeof(double), cudaMemcpyDeviceToHost, b->stream),
+           "cudaMemcpyAsync D2H");
   CK(cudaStreamSynchronize(b->stream), "sync");
   return SHASTA_OK;
 }
@@ -956,9 +948,9 @@ shasta_status shasta_batch_totals(shasta_batch* b, int id, double out[5]) {
   if (!e) return b ? fail(b, SHASTA_ENOTFOUND, "unknown event id") : SHASTA_EINVAL;
   if (!out) return fail(b, SHASTA_EINVAL, "out is NULL");
   DeviceGuard dg(b->device);
-  CK(launch_totals(view_of(b, *e, b->cur), e->ncell, 1, b->partials, b->d_tot, b->stream), "totals");
-  CK(cudaMemcpyAsync(b->h_small, b->d_tot, 5 * sizeof(double), cudaMemcpyDeviceToHost, b->stream),
-     "memcpy totals");
+  CK(launch_totals(view_of(b, *e, b->cur), e->ncell, 1, b->partials,
+                   (unsigned*)(b->d_count + b->o.max_events + 2), b->h_small, b->stream),
+     "totals");
   CK(cudaStreamSynchronize(b->stream), "sync");
   for (int k = 0; k < 5; ++k) out[k] = b->h_small[k];
   return SHASTA_OK;

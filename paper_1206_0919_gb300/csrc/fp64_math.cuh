@@ -36,6 +36,38 @@ __device__ __forceinline__ double scale(double x) {
   return __hiloint2double(hi(x) + (K << 20), __double2loint(x));
 }
 
+__device__ __forceinline__ long long bits(double x) { return __double_as_longlong(x); }
+
+// float -> double and back by the bit patterns (the conversion instructions
+// go through the double pipe: one of its slots each).  Zeros and normal
+// numbers; the rest, and what rounds to a subnormal float, by the instruction
+// (out of line: inlined, the compiler predicates it and every cell pays).
+static __device__ __noinline__ double widen_rest(float f) { return (double)f; }
+static __device__ __noinline__ float narrow_rest(double x) { return (float)x; }
+__device__ __forceinline__ double widen(float f) {
+  const unsigned u = __float_as_uint(f), a = u & 0x7fffffffu;
+  if (a - 0x00800000u < 0x7f000000u || a == 0u)
+    return __hiloint2double((int)((u & 0x80000000u) | (a ? (a >> 3) + 0x38000000u : 0u)), (int)(u << 29));
+  return widen_rest(f);
+}
+__device__ __forceinline__ double widen(double x) { return x; }
+template <class T>
+__device__ __forceinline__ T narrow(double x) {
+  if constexpr (sizeof(T) == 8) {
+    return x;
+  } else {
+    const unsigned a = mag(x);
+    const unsigned long long b = (unsigned long long)bits(x) & 0x7fffffffffffffffull;
+    const bool z = is_zero(x);
+    if (a - 0x38100000u < 0x47e00000u - 0x38100000u || z) {  // 2^-126 <= |x| < 2^127, or zero
+      const unsigned long long r = b + 0x0fffffffull + ((b >> 29) & 1ull);  // to nearest even
+      const unsigned f = z ? 0u : (unsigned)(r >> 29) - (896u << 23);
+      return __uint_as_float(f | ((unsigned)hi(x) & 0x80000000u));
+    }
+    return narrow_rest(x);
+  }
+}
+
 // 1/y to about an ulp, y normal and well inside the range.  For a
 // significand of ones the quotients of the correction below can be ties that
 // only the rounded-up reciprocal breaks the right way: there r is a power of
@@ -66,8 +98,8 @@ __device__ __forceinline__ double sqrt_raw(double x) {
 
 // the IEEE operators, out of line: inlined, the compiler predicates them and
 // every cell pays
-__device__ __noinline__ double ieee_div(double a, double y) { return a / y; }
-__device__ __noinline__ double ieee_sqrt(double x) { return ::sqrt(x); }
+static __device__ __noinline__ double ieee_div(double a, double y) { return a / y; }
+static __device__ __noinline__ double ieee_sqrt(double x) { return ::sqrt(x); }
 
 __device__ __forceinline__ double div(double a, double y) {
   if (within<-400, 400>(y) && (within<-500, 500>(a) || is_zero(a))) {

@@ -95,29 +95,31 @@ struct EosParams {
 };
 
 // Auxiliary kernels (aux.cu).  `is32` selects float (1) or double (0) storage.
-cudaError_t launch_from_f64(const double* src, void* dst, long long dstride, size_t n, int is32,
-                            cudaStream_t s);
-cudaError_t launch_to_f64(const void* src, long long sstride, double* dst, size_t n, int is32,
-                          cudaStream_t s);
+// Conversions between five arrays of doubles and a state (get: NULL arrays are
+// left out).
+cudaError_t launch_set_cons(const double* const in[5], const FieldView& out, size_t n, int is32, cudaStream_t s);
+cudaError_t launch_get_cons(const FieldView& in, double* const out[5], size_t n, int is32, cudaStream_t s);
 cudaError_t launch_prim2cons(const double* const prim[5], const FieldView& cons, size_t n,
                              int is32, EosParams eos, cudaStream_t s);
 cudaError_t launch_recover(const FieldView& cons, double* const prim[6], size_t n, int is32,
                            EosParams eos, cudaStream_t s);
-// Counts cells with non-finite values, E < 0 or |M| >= E (cons) or e < 0,
-// n < 0, |v| >= 1 (prims) into *count (device).
-cudaError_t launch_check_cons(const double* const f[5], size_t n, unsigned long long* count,
-                              cudaStream_t s);
-cudaError_t launch_check_prims(const double* const f[5], size_t n, unsigned long long* count,
-                               cudaStream_t s);
+// Number of cells with non-finite values, E < 0 or |M| >= E (cons) or e < 0,
+// n < 0, |v| >= 1 (prims) into *result (device or pinned host memory).
+// scratch: two device words, zero before the first use and left zero; one
+// check at a time per scratch.
+cudaError_t launch_check(bool prims, const double* const f[5], size_t n, unsigned long long* scratch,
+                         unsigned long long* result, cudaStream_t s);
 // Totals: per-block partial sums into `partials` (5 * nblocks doubles, device
-// scratch), then one block sums them in fixed order into out[5] (device).
+// scratch), which the last block sums in fixed order into out[5] (device or
+// pinned host memory).  ticket: one device word, zero before the first use and
+// left zero.
 int totals_blocks(size_t n);
-cudaError_t launch_totals(const FieldView& f, size_t n, int is32, double* partials, double* out,
+cudaError_t launch_totals(const FieldView& f, size_t n, int is32, double* partials, unsigned* ticket, double* out,
                           cudaStream_t s);
-// The same two-pass totals with an explicit chunk per block and block count
-// nb (partials: 5 * nb doubles of scratch).
-cudaError_t launch_totals_chunked(const FieldView& f, size_t n, int is32, size_t chunk, int nb,
-                                  double* partials, double* out, cudaStream_t s);
+// The same totals of a double state with an explicit chunk per block and block
+// count nb (partials: 5 * nb doubles of scratch), without a ticket.
+cudaError_t launch_totals_chunked(const FieldView& f, size_t n, size_t chunk, int nb, double* partials, double* out,
+                                  cudaStream_t s);
 // Frozen ghost store: for each axis a block [side][layer][field][plane].
 size_t frozen_elems(int nx, int ny, int nz);
 size_t frozen_axis_offset(int nx, int ny, int nz, int axis);

@@ -18,10 +18,11 @@ using namespace shasta;
 
 namespace {
 
-// One partial sum per block and field.  Each block sums a fixed run of cells,
+// One partial sum per block and field.  A block sums at most this many cells,
 // so the array bounds the number of cells one call can take.
 constexpr size_t kCellsPerBlock = SHASTA_TOTALS_NOALLOC_CELLS_PER_BLOCK;
 constexpr int kMaxBlocks = (int)(SHASTA_TOTALS_NOALLOC_MAX_CELLS / kCellsPerBlock);
+constexpr size_t kEvenBlocks = 4 * 152;
 static_assert((size_t)kMaxBlocks * kCellsPerBlock == SHASTA_TOTALS_NOALLOC_MAX_CELLS,
               "the cell limit is a whole number of blocks");
 
@@ -61,8 +62,13 @@ extern "C" shasta_status shasta_totals_noalloc(const double* E, const double* Mx
   }
   // Every partial the final pass reads is written by the first pass of the
   // same call, so nothing left in the array by an earlier call is used.
-  int nb = (int)((n + kCellsPerBlock - 1) / kCellsPerBlock);
-  cudaError_t e = launch_totals_chunked(f, n, 0, kCellsPerBlock, nb, scratch, out,
+  // The sums are bound by the double pipe (5 additions per cell), so they want
+  // every SM evenly filled: four blocks on each of 152, or whole 8192-cell
+  // blocks where those are more.
+  size_t chunk = (n + kEvenBlocks - 1) / kEvenBlocks;
+  chunk = chunk > kCellsPerBlock ? kCellsPerBlock : (chunk < 256 ? 256 : chunk);
+  int nb = (int)((n + chunk - 1) / chunk);
+  cudaError_t e = launch_totals_chunked(f, n, chunk, nb, scratch, out,
                                         static_cast<cudaStream_t>(stream));
   return e == cudaSuccess ? SHASTA_OK : SHASTA_ECUDA;
 }

@@ -26,8 +26,7 @@ using shasta::RangeAlloc;
 using shasta::batch_add_enqueue;
 using shasta::batch_extract_enqueue;
 using shasta::batch_remove_enqueue;
-using shasta::launch_check_cons;
-using shasta::launch_check_prims;
+using shasta::launch_check;
 
 namespace {
 
@@ -145,7 +144,7 @@ struct shasta_server {
   char* out_base = nullptr;
   RangeAlloc in_arena{256}, out_arena{256};
   Bounce bounce;  // the deliverer's
-  // input scans of staged events: device counters and their pinned copies
+  // input scans of staged events: device scratch and the pinned results
   unsigned long long* d_chk = nullptr;
   unsigned long long* h_chk = nullptr;
   bool chk_used[kMaxStaged] = {};
@@ -387,14 +386,9 @@ bool stage(shasta_server* s) {
     if (e == cudaSuccess)
       e = cudaMemcpyAsync(d, j->in.data(), 5 * j->ncell * sizeof(double), cudaMemcpyHostToDevice,
                           s->copy);
-    if (e == cudaSuccess) e = cudaMemsetAsync(s->d_chk + c, 0, sizeof(unsigned long long), s->copy);
     if (e == cudaSuccess)
-      e = j->ev.kind == SHASTA_STATE_PRIMITIVE
-              ? launch_check_prims(f, (size_t)j->ncell, s->d_chk + c, s->copy)
-              : launch_check_cons(f, (size_t)j->ncell, s->d_chk + c, s->copy);
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(s->h_chk + c, s->d_chk + c, sizeof(unsigned long long),
-                          cudaMemcpyDeviceToHost, s->copy);
+      e = launch_check(j->ev.kind == SHASTA_STATE_PRIMITIVE, f, (size_t)j->ncell, s->d_chk + 2 * c, s->h_chk + c,
+                       s->copy);
     if (e == cudaSuccess) e = cudaEventRecord(j->in_ready, s->copy);
     s->staged.push_back(j);
     if (!cuda_ok(s, e, "copy in")) return false;
@@ -640,7 +634,8 @@ shasta_status shasta_server_create(const shasta_server_opts* o, shasta_server** 
     return bail(ce == cudaErrorMemoryAllocation ? SHASTA_ENOMEM : SHASTA_ECUDA,
                 std::string("staging: ") + cudaGetErrorString(ce));
   ce = bounce_init(s->bounce);
-  if (ce == cudaSuccess) ce = cudaMalloc((void**)&s->d_chk, kMaxStaged * sizeof(unsigned long long));
+  if (ce == cudaSuccess) ce = cudaMalloc((void**)&s->d_chk, 2 * kMaxStaged * sizeof(unsigned long long));
+  if (ce == cudaSuccess) ce = cudaMemset(s->d_chk, 0, 2 * kMaxStaged * sizeof(unsigned long long));
   if (ce == cudaSuccess) ce = cudaMallocHost((void**)&s->h_chk, kMaxStaged * sizeof(unsigned long long));
   for (int p = 0; p < 2 && ce == cudaSuccess; ++p)
     ce = cudaEventCreateWithFlags(&s->iter_done[p], cudaEventDisableTiming);

@@ -18,10 +18,12 @@
 // About 240 double operations per cell are left (the streaming kernel executes
 // 641).  Shared-memory traffic and the block barriers between stages hide
 // behind the double pipe.
-// MEASURED
+// Measured, streaming -> here (us a sweep): 64^3 507 -> 151, 143 x 129 x 151
+// 3588 -> 1497, 200^3 8925 -> 4306; the double pipe is 83% busy (85-87% is the
+// most any kernel here reaches, with no barriers in it).
 #pragma once
 
-#include "fp64_math.cuh"
+#include "eos64.cuh"
 #include "lines_plan.h"
 #include "sweep.cuh"
 
@@ -37,7 +39,7 @@ struct LineArgs {
 };
 
 
-__device__ __forceinline__ long long bits(double x) { return __double_as_longlong(x); }
+using f64::bits;
 
 // Limiter of Sec. 3, s max(0, min(s dhp, |aph|, s dhm)), by the bit patterns:
 // nonnegative doubles order as integers.  Infinities and NaN take the
@@ -59,58 +61,6 @@ __device__ __forceinline__ double times_eta(double x, double eta, int k) {
   if (f64::is_zero(x)) return x;  // (eta >= 0)
   if (k == 0 || f64::mag(x) - 0x04000000u >= 0x7ff00000u - 0x04000000u) return eta * x;
   return __hiloint2double(f64::hi(x) - (k << 20), __double2loint(x));
-}
-
-// p(e) of the table and its fixed point (table_p64, eos_table_solve of
-// sweep.cuh), with the reciprocal of the spacing kept.
-__device__ __forceinline__ double table_at(const EosTable& T, double rde, double e) {
-  const bool z = f64::is_zero(e);
-  double x;
-  if ((z || f64::within<-500, 500>(e)) && f64::within<-400, 400>(T.de)) {
-    const double q = e * rde;
-    x = z ? q : fma(fma(-T.de, q, e), rde, q);
-  } else {
-    x = e / T.de;
-  }
-  int k = __double2int_rd(x);
-  k = k < 0 ? 0 : (k > T.n - 2 ? T.n - 2 : k);
-  const double f = x - (double)k;
-  const double a = __ldg(T.p64 + k), b = __ldg(T.p64 + k + 1);
-  return a + f * (b - a);
-}
-__device__ __forceinline__ void table_solve(double E, double M, const EosTable& T, double& p) {
-  const double rde = f64::recip_raw(T.de);
-  double v = f64::div(M, E + table_at(T, rde, E));
-  for (int it = 0; it < 200; ++it) {
-    const double vn = f64::div(M, E + table_at(T, rde, E - M * v));
-    const double d = vn - v;
-    v = vn;
-    if ((bits(d) & ~(1ll << 63)) <= bits(1e-14)) break;
-  }
-  p = table_at(T, rde, E - M * v);
-}
-
-// Root of the EoS for a cell inside the safe range (eos_solve of sweep.cuh).
-template <int EOS>
-__device__ __forceinline__ double pressure(double E, double M, double B, double ec) {
-  const double m3 = (3.0 * M) * M;
-  const double s = f64::sqrt_raw((f64::scale<2>(E) * E) - m3);
-  const double EM = (E - M) * (E + M);
-  const double se = s + E;
-  const double pa = f64::quot_raw(EM, se, f64::recip_raw(se));
-  if constexpr (EOS == EOS_BAG) {
-    if (3.0 * pa <= ec) return pa;
-    if (E > ec) {
-      const double r = (4.0 * (E - B)) * (E - B) - m3;
-      if (r >= 0.0) {
-        const double sb = f64::sqrt(r);
-        const double eb = f64::div(3.0 * EM - (4.0 * B) * E, sb + (E - 2.0 * B));
-        if (eb > ec) return f64::div(eb - 4.0 * B, 3.0);
-      }
-    }
-    return f64::div(M * M, E - ec) - E;
-  }
-  return pa;
 }
 
 // m/h for h in [2^-401, 2^401) and any |m| <= h, m != 0: the momentum in the
@@ -148,11 +98,11 @@ __device__ __forceinline__ unsigned recover(double E, double m1, double m2, doub
   if (f64::hi(E) > 0 && f64::within<-400, 400>(E) && (still || f64::within<-940, 810>(M2))) {
     const double M = still ? 0.0 : f64::sqrt_raw(M2);
     if (bits(M) <= bits(omd * E)) {
-      if constexpr (EOS == EOS_TABLE) {
-        table_solve(E, M, T, p);
-      } else {
-        p = pressure<EOS>(E, M, B, ec);
-      }
+      double e;
+      if constexpr (EOS == EOS_TABLE)
+        f64::table_solve(E, M, T, e, p);
+      else
+        f64::closed_root<EOS>(E, M, B, ec, e, p);
       const double h = E + p;
       if (f64::is_zero(m1))
         w = m1;  // (h > 0)
