@@ -51,6 +51,7 @@
 
 #include <type_traits>
 
+#include "fp64_math.cuh"
 #include "sweep.cuh"
 
 namespace shasta {
@@ -326,9 +327,10 @@ constexpr int REC_F32 = 0, REC_DF = 1, REC_F64 = 2;
 // REC_F64: velocity along the sweep and pressure of one cell, every
 // operation in double (IEEE division and square root) on the float state;
 // the same closed forms as rec32 below.  omd = 1 - delta in double.
+// This form, with the IEEE operators, for the cells rec64 leaves out.
 template <int EOS>
-__device__ __forceinline__ unsigned rec64(float Ef, float mxf, float myf, float mzf, float m1f,
-                                          double omd, double B, double ec, float& w, float& p) {
+__device__ __noinline__ unsigned rec64_rest(float Ef, float mxf, float myf, float mzf, float m1f,
+                                            double omd, double B, double ec, float& w, float& p) {
   const double E = Ef, mx = mxf, my = myf, mz = mzf;
   unsigned clamped = 0;
   double M2 = fma(mx, mx, fma(my, my, mz * mz));
@@ -362,6 +364,52 @@ __device__ __forceinline__ unsigned rec64(float Ef, float mxf, float myf, float 
     clamped = 1;
   }
   return clamped;
+}
+
+// Whether |M| exceeds (1 - delta) E (out of line: asked near |v| = 1 only).
+static __device__ __noinline__ bool rec64_over(double E, double M2, double omd) {
+  const double lim = omd * E;
+  return !(M2 <= lim * lim);
+}
+
+// The same bits for a physical, unclamped cell with a normal E: bound by the
+// double pipe (2 operations per SM and clock), so the quotients and the root
+// are the short ones, comparisons and conversions integer operations, and the
+// clamp is compared exactly only within 1/32 of E^2: 28 double operations for
+// the ideal gas instead of about 65.
+template <int EOS>
+__device__ __forceinline__ unsigned rec64(float Ef, float mxf, float myf, float mzf, float m1f,
+                                          double omd, double B, double ec, float& w, float& p) {
+  if (__float_as_uint(Ef) - 0x00800000u < 0x7f000000u) {
+    const double E = f64::widen(Ef), mx = f64::widen(mxf), my = f64::widen(myf), mz = f64::widen(mzf);
+    const double M2 = fma(mx, mx, fma(my, my, mz * mz));
+    const double E2 = E * E;
+    if (!((f64::hi(M2) > f64::hi(E2) - 0x8000 || f64::hi(omd) < 0x3fefae15) && rec64_over(E, M2, omd))) {
+      double D = fma(E, E, -M2);
+      if (f64::hi(D) < 0) D = 0.0;
+      double pp;
+      if constexpr (EOS == EOS_BAG) {
+        const double D3 = 3.0 * D;
+        const bool bag = f64::bits(D3) > f64::bits(ec * fma(2.0, E, ec));
+        const double b = bag ? B : 0.0;
+        const double q = fma(-4.0, b, E);
+        const double r = fma(3.0, D, fma(q, q, -12.0 * (b * b)));
+        const double s = f64::sqrt(f64::hi(r) < 0 ? 0.0 : r);
+        pp = f64::div(fma(-(4.0 / 3.0) * b, E, D), fma(-2.0, b, E + s)) - (4.0 / 3.0) * b;
+        if (bag && !(E > ec && r >= 0.0 && fma(3.0, pp, 4.0 * B) > ec)) pp = f64::div(M2, E - ec) - E;
+      } else {
+        const double s = f64::sqrt_raw(fma(3.0, D, E2));
+        const double se = E + s;
+        pp = f64::quot_raw(D, se, f64::recip_raw(se));
+      }
+      const double h = E + pp;
+      const double m = f64::widen(m1f);
+      w = m1f == 0.0f ? m1f : f64::narrow<float>(f64::quot_raw(m, h, f64::recip_raw(h)));
+      p = f64::narrow<float>(pp);
+      return 0;
+    }
+  }
+  return rec64_rest<EOS>(Ef, mxf, myf, mzf, m1f, omd, B, ec, w, p);
 }
 
 // Velocity along the sweep and pressure of one cell, FP32 (REC_DF: D in
