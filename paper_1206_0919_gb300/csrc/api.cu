@@ -86,6 +86,7 @@ struct shasta_ctx {
   LinesPlan lines[3] = {};  // FP64: whole-line sweep of each axis (B 0: none)
   int force_tile = -1, force_lines = 0;
   bool stream_only = false;
+  bool chain = false;     // overlap launches at their ends (not inside a graph)
   bool tuned = false;     // autotuned launch choice below is valid
   bool tune_tile[3] = {false, false, false};
   int tune_var[3] = {0, 0, 0};
@@ -425,15 +426,15 @@ shasta_status prepare_ranges(shasta_ctx* c) {
 }
 
 cudaError_t launch_tile(shasta_ctx* c, int axis, const SweepParams& P) {
-  if (c->o.precision == SHASTA_FP64) return launch_lines_f64(P, c->lines[axis], axis, c->eos.kind, c->stream);
+  if (c->o.precision == SHASTA_FP64) return launch_lines_f64(P, c->lines[axis], axis, c->eos.kind, c->chain, c->stream);
   const TilePlan& t = c->tile[axis];
   const bool bag = c->eos.kind == SHASTA_EOS_BAG;
   if (c->o.precision == SHASTA_MIXED)
-    return (bag ? launch_tile_mixed_bag : launch_tile_mixed_ideal)(P, t, axis, c->sm_count, c->stream);
+    return (bag ? launch_tile_mixed_bag : launch_tile_mixed_ideal)(P, t, axis, c->sm_count, c->chain, c->stream);
   if (c->o.precision == SHASTA_MIXED_FP64)
-    return (bag ? launch_tile_mixed64_bag : launch_tile_mixed64_ideal)(P, t, axis, c->sm_count, c->stream);
-  if (c->eos.kind == SHASTA_EOS_TABLE) return launch_tile_f32_table(P, t, axis, c->sm_count, c->stream);
-  return (bag ? launch_tile_f32_bag : launch_tile_f32_ideal)(P, t, axis, c->sm_count, c->stream);
+    return (bag ? launch_tile_mixed64_bag : launch_tile_mixed64_ideal)(P, t, axis, c->sm_count, c->chain, c->stream);
+  if (c->eos.kind == SHASTA_EOS_TABLE) return launch_tile_f32_table(P, t, axis, c->sm_count, c->chain, c->stream);
+  return (bag ? launch_tile_f32_bag : launch_tile_f32_ideal)(P, t, axis, c->sm_count, c->chain, c->stream);
 }
 
 // Cuts the lines of an axis into tiles (FP64: into blocks of whole lines) and
@@ -1007,7 +1008,10 @@ shasta_status shasta_step(shasta_ctx* c, int nsteps) {
       nsteps -= 6;
       continue;
     }
-    CK(launch_step(c, (int)(c->steps % 6)), "sweep launch");
+    c->chain = true;
+    const cudaError_t le = launch_step(c, (int)(c->steps % 6));
+    c->chain = false;
+    CK(le, "sweep launch");
     ++c->steps;
     --nsteps;
   }

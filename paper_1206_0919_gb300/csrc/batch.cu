@@ -68,7 +68,7 @@ struct shasta_batch {
   int nlive = 0;
   long long used = 0;
   EvDesc* d_desc = nullptr;
-  unsigned long long* d_count = nullptr;  // per slot clamp counters; from [max_events]: check scratch (2), totals ticket
+  unsigned long long* d_count = nullptr;  // clamp counter per slot; from [max_events]: check scratch (2), totals ticket
   int* d_plan = nullptr;
   size_t plan_cap = 0;  // ints
   // work-list uploads go through two pinned buffers used in turn, so that a

@@ -17,7 +17,8 @@ cudaError_t launch_sweep_f64(const SweepParams& P, int axis, int eos, cudaStream
 // FP64 sweeps on whole lines in shared memory (bitwise the streaming ones);
 // prepare_lines_f64 before the first launch or capture.
 cudaError_t prepare_lines_f64(int axis, int eos, const LinesPlan& t);
-cudaError_t launch_lines_f64(const SweepParams& P, const LinesPlan& t, int axis, int eos, cudaStream_t s);
+cudaError_t launch_lines_f64(const SweepParams& P, const LinesPlan& t, int axis, int eos, bool chain,
+                             cudaStream_t s);
 cudaError_t launch_sweep_f32(const SweepParams& P, int axis, int eos, cudaStream_t s);
 cudaError_t launch_sweep_mixed(const SweepParams& P, int axis, int eos, cudaStream_t s);
 cudaError_t launch_sweep_mixed64(const SweepParams& P, int axis, int eos, cudaStream_t s);
@@ -51,7 +52,7 @@ int sweep_warps_per_block_mixed64();
 // Tiled FP32 / MIXED sweeps (tile_*.cu): bitwise the streaming ones, for the
 // sizes where those are bound by their serial chain.  prepare_* sets the
 // shared-memory attribute of one (axis, shape) kernel and reports its resident
-// blocks per SM (before the first launch or capture).
+// blocks per SM (before the first launch or capture).  chain: chain.cuh.
 cudaError_t prepare_tile_f32_ideal(int axis, int shape, int* blocks_per_sm);
 cudaError_t prepare_tile_f32_bag(int axis, int shape, int* blocks_per_sm);
 cudaError_t prepare_tile_f32_table(int axis, int shape, int* blocks_per_sm);
@@ -59,14 +60,19 @@ cudaError_t prepare_tile_mixed_ideal(int axis, int shape, int* blocks_per_sm);
 cudaError_t prepare_tile_mixed_bag(int axis, int shape, int* blocks_per_sm);
 cudaError_t prepare_tile_mixed64_ideal(int axis, int shape, int* blocks_per_sm);
 cudaError_t prepare_tile_mixed64_bag(int axis, int shape, int* blocks_per_sm);
-cudaError_t launch_tile_f32_ideal(const SweepParams& P, const TilePlan& t, int axis, int sm_count, cudaStream_t s);
-cudaError_t launch_tile_f32_bag(const SweepParams& P, const TilePlan& t, int axis, int sm_count, cudaStream_t s);
-cudaError_t launch_tile_f32_table(const SweepParams& P, const TilePlan& t, int axis, int sm_count, cudaStream_t s);
-cudaError_t launch_tile_mixed_ideal(const SweepParams& P, const TilePlan& t, int axis, int sm_count, cudaStream_t s);
-cudaError_t launch_tile_mixed_bag(const SweepParams& P, const TilePlan& t, int axis, int sm_count, cudaStream_t s);
-cudaError_t launch_tile_mixed64_ideal(const SweepParams& P, const TilePlan& t, int axis, int sm_count,
+cudaError_t launch_tile_f32_ideal(const SweepParams& P, const TilePlan& t, int axis, int sm_count, bool chain,
+                                  cudaStream_t s);
+cudaError_t launch_tile_f32_bag(const SweepParams& P, const TilePlan& t, int axis, int sm_count, bool chain,
+                                cudaStream_t s);
+cudaError_t launch_tile_f32_table(const SweepParams& P, const TilePlan& t, int axis, int sm_count, bool chain,
+                                  cudaStream_t s);
+cudaError_t launch_tile_mixed_ideal(const SweepParams& P, const TilePlan& t, int axis, int sm_count, bool chain,
+                                    cudaStream_t s);
+cudaError_t launch_tile_mixed_bag(const SweepParams& P, const TilePlan& t, int axis, int sm_count, bool chain,
+                                  cudaStream_t s);
+cudaError_t launch_tile_mixed64_ideal(const SweepParams& P, const TilePlan& t, int axis, int sm_count, bool chain,
                                       cudaStream_t s);
-cudaError_t launch_tile_mixed64_bag(const SweepParams& P, const TilePlan& t, int axis, int sm_count,
+cudaError_t launch_tile_mixed64_bag(const SweepParams& P, const TilePlan& t, int axis, int sm_count, bool chain,
                                     cudaStream_t s);
 // Batched FP32 / MIXED sweeps (one launch over the work list L, all along
 // `axis`); prepare_* as above for the batched kernels.

@@ -2,6 +2,7 @@
 // -fmad=false and IEEE division / square root so that the arithmetic is the
 // plain double-precision evaluation of each expression in source order.
 #include "kernels.h"
+#include "chain.cuh"
 #include "sweep_lines64.cuh"
 
 #include <math.h>
@@ -35,7 +36,8 @@ cudaError_t prepare_lines_f64(int axis, int eos, const LinesPlan& t) {
                               (int)kLinesSmem);
 }
 
-cudaError_t launch_lines_f64(const SweepParams& P, const LinesPlan& t, int axis, int eos, cudaStream_t s) {
+cudaError_t launch_lines_f64(const SweepParams& P, const LinesPlan& t, int axis, int eos, bool chain,
+                             cudaStream_t s) {
   if (P.plane <= 0) return cudaSuccess;
   if (t.B < 1 || P.n < NG) return cudaErrorInvalidValue;
   const int np = P.n + 2 * NG;
@@ -48,8 +50,8 @@ cudaError_t launch_lines_f64(const SweepParams& P, const LinesPlan& t, int axis,
   int ex;
   if (frexp(P.eta, &ex) == 0.5 && ex <= 0 && ex > -60) A.eta_exp = 1 - ex;
   void* args[] = {const_cast<SweepParams*>(&P), &A};
-  return cudaLaunchKernel(lines_kernel_of(eos, axis), dim3((unsigned)((P.plane + t.B - 1) / t.B)),
-                          dim3(t.threads), args, t.smem, s);
+  return launch_sweep_kernel(lines_kernel_of(eos, axis), dim3((unsigned)((P.plane + t.B - 1) / t.B)),
+                          dim3(t.threads), args, t.smem, chain, s);
 }
 
 cudaError_t launch_sweep_f64(const SweepParams& P, int axis, int eos, cudaStream_t s) {

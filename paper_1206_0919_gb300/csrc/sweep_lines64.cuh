@@ -23,6 +23,7 @@
 // most any kernel here reaches, with no barriers in it).
 #pragma once
 
+#include "chain.cuh"
 #include "eos64.cuh"
 #include "lines_plan.h"
 #include "sweep.cuh"
@@ -165,6 +166,7 @@ __global__ void __launch_bounds__(kLinesMaxThreads) sweep_lines_kernel(SweepPara
     return __hiloint2double(f64::hi(x) ^ (f ? 0x80000000 : 0), __double2loint(x));
   };
 
+  chain_begin();
   // ---- the old state, ghosts included
   each(-NG, n + NG, [&](int j, int l) {
     const long long t = t0 + l;

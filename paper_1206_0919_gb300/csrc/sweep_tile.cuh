@@ -37,6 +37,7 @@
 //    Two buffers: the next tile is copied while one is computed.
 #pragma once
 
+#include "chain.cuh"
 #include "sweep_fast.cuh"
 
 namespace shasta {
@@ -404,6 +405,7 @@ __global__ void __launch_bounds__(Lay<AXIS, C, XL>::WARPS * 32, MINB)
     }
   };
 
+  chain_begin();
   if (seg < ntile) issue(seg, k, buf0);
   cp_commit();
   int cur = 0;

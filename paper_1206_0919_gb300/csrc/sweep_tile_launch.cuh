@@ -3,6 +3,7 @@
 // including unit.
 #pragma once
 
+#include "chain.cuh"
 #include "kernels.h"
 #include "sweep_tile.cuh"
 
@@ -66,7 +67,7 @@ cudaError_t prepare(int axis, int shape, int* blocks_per_sm) {
 }
 
 template <int EOS, int REC>
-cudaError_t launch(const SweepParams& P, const TilePlan& t, int axis, int sm_count, cudaStream_t s) {
+cudaError_t launch(const SweepParams& P, const TilePlan& t, int axis, int sm_count, bool chain, cudaStream_t s) {
   if (P.plane <= 0) return cudaSuccess;
   const Kern k = lookup<EOS, REC>(axis, t.shape);
   if (!k.fun || t.blocks_per_sm < 1 || t.ntile < 1) return cudaErrorInvalidValue;
@@ -78,7 +79,8 @@ cudaError_t launch(const SweepParams& P, const TilePlan& t, int axis, int sm_cou
   const long long need = axis == 0 ? (tiles + k.warps - 1) / k.warps : tiles;  // x: one tile per warp
   const long long wave = (long long)sm_count * t.blocks_per_sm;
   void* args[] = {const_cast<SweepParams*>(&P), &A};
-  return cudaLaunchKernel(k.fun, dim3((unsigned)(need < wave ? need : wave)), dim3(k.warps * 32), args, k.smem, s);
+  return launch_sweep_kernel(k.fun, dim3((unsigned)(need < wave ? need : wave)), dim3(k.warps * 32), args, k.smem,
+                             chain, s);
 }
 
 }  // namespace tile

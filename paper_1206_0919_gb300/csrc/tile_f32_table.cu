@@ -7,8 +7,9 @@ cudaError_t prepare_tile_f32_table(int axis, int shape, int* blocks_per_sm) {
   return tile::prepare<EOS_TABLE, fast::REC_F32>(axis, shape, blocks_per_sm);
 }
 
-cudaError_t launch_tile_f32_table(const SweepParams& P, const TilePlan& t, int axis, int sm_count, cudaStream_t s) {
-  return tile::launch<EOS_TABLE, fast::REC_F32>(P, t, axis, sm_count, s);
+cudaError_t launch_tile_f32_table(const SweepParams& P, const TilePlan& t, int axis, int sm_count, bool chain,
+                                  cudaStream_t s) {
+  return tile::launch<EOS_TABLE, fast::REC_F32>(P, t, axis, sm_count, chain, s);
 }
 
 }  // namespace shasta
