@@ -518,27 +518,31 @@ void drop_graph(shasta_ctx* c) {
   c->graph = nullptr;
 }
 
-// Time of `reps` sweeps of axis with parameters P, on tiles or streamed
-// (after `warm` untimed ones), from the current buffer into the other one.
-cudaError_t time_choice(shasta_ctx* c, int axis, bool tile, SweepParams P, int warm, int reps,
-                        cudaEvent_t e0, cudaEvent_t e1, float& ms) {
+// Time of one sweep of axis with parameters P, on tiles or streamed, from the
+// current buffer into the other one: one launch after an untimed one (two
+// runs of a choice differ by 0.1% at 0.1 ms and more), five of short ones.
+cudaError_t time_choice(shasta_ctx* c, int axis, bool tile, SweepParams P, cudaEvent_t e0, cudaEvent_t e1, float& ms) {
   P.clamp_count = nullptr;  // trial sweeps are no steps: their clamps do not count
-  auto go = [&] { return tile ? launch_tile(c, axis, P) : launch_params(c, axis, P); };
-  cudaError_t ce = cudaSuccess;
-  for (int r = 0; r < warm && ce == cudaSuccess; ++r) ce = go();
-  if (ce == cudaSuccess) ce = cudaEventRecord(e0, c->stream);
-  for (int r = 0; r < reps && ce == cudaSuccess; ++r) ce = go();
-  if (ce == cudaSuccess) ce = cudaEventRecord(e1, c->stream);
-  if (ce == cudaSuccess) ce = cudaEventSynchronize(e1);
-  if (ce == cudaSuccess) ce = cudaEventElapsedTime(&ms, e0, e1);
+  cudaError_t ce = tile ? launch_tile(c, axis, P) : launch_params(c, axis, P);
+  for (int reps = 1; reps <= 5 && ce == cudaSuccess; reps += 4) {
+    ce = cudaEventRecord(e0, c->stream);
+    for (int r = 0; r < reps && ce == cudaSuccess; ++r)
+      ce = tile ? launch_tile(c, axis, P) : launch_params(c, axis, P);
+    if (ce == cudaSuccess) ce = cudaEventRecord(e1, c->stream);
+    if (ce == cudaSuccess) ce = cudaEventSynchronize(e1);
+    if (ce == cudaSuccess) ce = cudaEventElapsedTime(&ms, e0, e1);
+    ms /= (float)reps;
+    if (ms > 0.2f) break;
+  }
   return ce;
 }
 
 // Times candidate launch choices per axis with repeated sweeps from the
 // current buffer into the other one (the state itself is not changed) and
 // keeps the fastest.  FP32 / MIXED: tiles (alone, untimed, where a warp's
-// streamed share is under kTileAlways), or the register variant and ranges of
-// one line group (no line is cut) or of 1/4 .. 3 ranges per resident warp.
+// streamed share is under kTileAlways), or ranges of one line group (no line is
+// cut) or of 1/2 .. 2 ranges per resident warp, and the best of them with the
+// other register variant.
 // FP64: nothing to time on whole lines in shared memory; else the line segment
 // length (the default one, 24 .. 128 cells, whole lines).  The choice does not change results.
 shasta_status autotune(shasta_ctx* c) {
@@ -551,7 +555,7 @@ shasta_status autotune(shasta_ctx* c) {
   CK(cudaEventCreate(&e1), "cudaEventCreate");
   shasta_status st = SHASTA_OK;
   const bool f64 = c->o.precision == SHASTA_FP64;
-  static const double shares[] = {0.25, 0.5, 1.0, 2.0, 3.0};
+  static const double shares[] = {0.5, 1.0, 2.0};
   static const long long segments[] = {24, 32, 48, 64, 100, 128};
   for (int axis = 0; axis < 3 && st == SHASTA_OK; ++axis) {
     const int n = axis == 0 ? c->g.nx : (axis == 1 ? c->g.ny : c->g.nz);
@@ -560,13 +564,15 @@ shasta_status autotune(shasta_ctx* c) {
     int bv = 0;
     long long br = f64 ? fp64_segment(c, axis) : n;
     bool bt = false;
+    float sbest = 1e30f;  // the best of the streaming choices, and its share (0: whole line groups)
+    double bsh = 0.0;
     if (f64 && c->lines[axis].B > 0) continue;
     if (c->tile[axis].shape >= 0) {
       if (c->force_tile >= 0 || stream_share(c, axis) < kTileAlways) {
         c->tune_tile[axis] = true;
         continue;
       }
-      const cudaError_t ce = time_choice(c, axis, true, sweep_params(c, axis, c->cur, 0, 1), 2, 4, e0, e1, best);
+      const cudaError_t ce = time_choice(c, axis, true, sweep_params(c, axis, c->cur, 0, 1), e0, e1, best);
       if (ce != cudaSuccess) {
         st = cuda_fail(c, ce, "autotune");
         break;
@@ -588,10 +594,14 @@ shasta_status autotune(shasta_ctx* c) {
         add(n);
       } else {
         const long long warps = (long long)c->sm_count * c->occ[c->eos.kind][axis][var];
-        add(n);
-        for (double sh : shares) {
-          const long long r = range_for(total, warps, sh);
-          if (r < total) add(r);
+        if (var == 1) {
+          add(bsh > 0.0 ? range_for(total, warps, bsh) : n);
+        } else {
+          add(n);
+          for (double sh : shares) {
+            const long long r = range_for(total, warps, sh);
+            if (r < total) add(r);
+          }
         }
       }
       for (int ci = 0; ci < nc && st == SHASTA_OK; ++ci) {
@@ -599,10 +609,17 @@ shasta_status autotune(shasta_ctx* c) {
         if (st != SHASTA_OK) break;
         float ms = 0;
         const cudaError_t ce = time_choice(c, axis, false, sweep_params(c, axis, c->cur, var, cands[ci]),
-                                           f64 ? 1 : 2, f64 ? 2 : 4, e0, e1, ms);
+                                           e0, e1, ms);
         if (ce != cudaSuccess) {
           st = cuda_fail(c, ce, "autotune");
           break;
+        }
+        if (!f64 && var == 0 && ms < sbest) {
+          sbest = ms;
+          bsh = 0.0;
+          for (double sh : shares)
+            if (cands[ci] != n && cands[ci] == range_for(total, (long long)c->sm_count * c->occ[c->eos.kind][axis][0], sh))
+              bsh = sh;
         }
         if (ms < best) {
           best = ms;
@@ -626,7 +643,7 @@ shasta_status autotune(shasta_ctx* c) {
         st = ensure_ranges(c, axis, br, bv);
         if (st != SHASTA_OK) break;
         float ms = 0;
-        const cudaError_t ce = time_choice(c, axis, false, sweep_params(c, axis, c->cur, bv, br), 2, 4, e0, e1, ms);
+        const cudaError_t ce = time_choice(c, axis, false, sweep_params(c, axis, c->cur, bv, br), e0, e1, ms);
         if (ce != cudaSuccess) {
           st = cuda_fail(c, ce, "autotune");
           break;

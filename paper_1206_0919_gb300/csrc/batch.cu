@@ -449,31 +449,44 @@ shasta_status autotune(shasta_batch* b) {
     float best = 1e30f;
     int bv = 0;
     long long br = b->tune_range[a];
-    for (int var = 0; var < 2 && st == SHASTA_OK; ++var)
-      for (double sh : shares) {
-        // share 0: whole line groups
-        const long long range = sh > 0 ? range_for(total, warp_slots(b, 0, a, var), sh) : 0;
-        cudaError_t ce = cudaSuccess;
-        for (const LaunchRec& L : recs)
-          if (ce == cudaSuccess) ce = launch_rec(b, L, b->cur, var, range);
-        if (ce == cudaSuccess) ce = cudaEventRecord(e0, b->stream);
-        for (int rep = 0; rep < 3 && ce == cudaSuccess; ++rep)
-          for (const LaunchRec& L : recs)
-            if (ce == cudaSuccess) ce = launch_rec(b, L, b->cur, var, range);
+    double bsh = 0.0;
+    // one sweep of every event per choice after an untimed one, five where
+    // that is short (two runs of a choice differ by 0.1% at 0.1 ms and more);
+    // the other register variant for the best share only.  Every trial is
+    // time taken from the batch's own steps: 32 sweeps an axis were a third
+    // of a 48-step batch, these are 10.
+    auto sweep_all = [&](int var, long long range) {
+      cudaError_t ce = cudaSuccess;
+      for (const LaunchRec& L : recs)
+        if (ce == cudaSuccess) ce = launch_rec(b, L, b->cur, var, range);
+      return ce;
+    };
+    auto trial = [&](int var, double sh) {
+      // share 0: whole line groups
+      const long long range = sh > 0 ? range_for(total, warp_slots(b, 0, a, var), sh) : 0;
+      cudaError_t ce = sweep_all(var, range);
+      float ms = 0;
+      for (int reps = 1; reps <= 5 && ce == cudaSuccess; reps += 4) {
+        ce = cudaEventRecord(e0, b->stream);
+        for (int r = 0; r < reps && ce == cudaSuccess; ++r) ce = sweep_all(var, range);
         if (ce == cudaSuccess) ce = cudaEventRecord(e1, b->stream);
         if (ce == cudaSuccess) ce = cudaEventSynchronize(e1);
-        float ms = 0;
         if (ce == cudaSuccess) ce = cudaEventElapsedTime(&ms, e0, e1);
-        if (ce != cudaSuccess) {
-          st = cuda_fail(b, ce, "autotune");
-          break;
-        }
-        if (ms < best) {
-          best = ms;
-          bv = var;
-          br = range;
-        }
+        ms /= (float)reps;
+        if (ms > 0.2f) break;
       }
+      if (ce != cudaSuccess) {
+        st = cuda_fail(b, ce, "autotune");
+      } else if (ms < best) {
+        best = ms;
+        bv = var;
+        br = range;
+        bsh = sh;
+      }
+    };
+    for (double sh : shares)
+      if (st == SHASTA_OK) trial(0, sh);
+    if (st == SHASTA_OK) trial(1, bsh);
     b->tune_var[a] = bv;
     b->tune_range[a] = br;
   }
