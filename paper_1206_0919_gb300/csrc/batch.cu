@@ -47,6 +47,8 @@ struct LaunchRec {
   size_t idx_off = 0, pre_off = 0, gpre_off = 0;  // event indices, position / group prefixes
   long long items = 0;   // (line group, position) pairs
   long long groups = 0;  // line groups
+  int variant = 0;       // register variant and positions per work range
+  long long range = 0;   // (0: whole line groups)
 };
 
 }  // namespace
@@ -87,11 +89,17 @@ struct shasta_batch {
   int sm_count = 152;
   int occ[3][3][2] = {};
   int wpb = 4;
-  // launch choice per axis: register variant and positions per work range
+  // launch choice per axis: register variant and ranges per resident warp
   bool tuned = false;
   long long force_range = -1;  // >= 0: work range of every axis (environment override; 0 = line groups)
   int tune_var[3] = {0, 0, 0};
-  long long tune_range[3] = {0, 0, 0};  // 0: whole line groups
+  double tune_share[3] = {0, 0, 0};  // ranges per resident warp; 0: whole line groups
+  // few small events: every event sweeps by the tiled kernels in launches of
+  // its own (resident blocks per SM of the kernels readied so far)
+  bool by_event = false;
+  bool trial = false;  // the autotuner's sweeps: no steps, their clamps do not count
+  bool tiles_off = false;
+  int tile_bps[2][3][kTileShapeCount] = {};
   // work lists of six consecutive steps (index (steps - plan_base) mod 6)
   bool plan_valid = false;
   int64_t bsteps = 0, plan_base = 0;
@@ -187,7 +195,7 @@ void model_choice(shasta_batch* b) {
   for (int a = 0; a < 3; ++a) {
     const long long warps = warp_slots(b, 0, a, 0);
     b->tune_var[a] = 0;
-    b->tune_range[a] = total_groups(b, a) >= 2 * warps ? 0 : range_for(total_positions(b, a), warps, 1.0);
+    b->tune_share[a] = total_groups(b, a) >= 2 * warps ? 0.0 : 1.0;
   }
 }
 
@@ -233,7 +241,7 @@ EvDesc desc_of(const shasta_batch* b, int i) {
     d.frozen[a] = e.frozen ? (const float*)e.frozen +
                                  frozen_axis_offset(e.g.nx, e.g.ny, e.g.nz, a)
                            : nullptr;
-  d.clamp_count = b->d_count + i;
+  d.clamp_count = b->trial ? nullptr : b->d_count + i;
   return d;
 }
 
@@ -323,6 +331,67 @@ LaunchRec make_list(const shasta_batch* b, std::vector<int> ids, int axis, int e
   return L;
 }
 
+// Sets the variants and range lengths of the launches of one sweep slot: for
+// a launch by itself `share` ranges per resident warp; several launches (both
+// EoS, or events at different phases) always take whole line groups.  Ranges
+// fill an SM with one long round of warps, and beside a second kernel that
+// round slows to less than half (192^3 ideal, 128^3 bag, 64^3 of each: 826 us a
+// step with ranges cut for both together, 559 with ranges for each, 397 with
+// line groups; 64^3 three of each 338 against 169; 160^3 of each 454 against
+// 374), while many short units let one kernel follow the other.
+void fit_ranges(const shasta_batch* b, std::vector<LaunchRec>& V, const int var[3], const double share[3]) {
+  for (LaunchRec& L : V) {
+    L.variant = var[L.axis];
+    if (b->force_range >= 0)
+      L.range = b->force_range;
+    else
+      L.range = share[L.axis] > 0.0 && V.size() == 1
+                    ? range_for(L.items, warp_slots(b, L.eos, L.axis, L.variant), share[L.axis])
+                    : 0;
+  }
+}
+
+// Few events of few positions take the tiled kernels, each event in launches
+// of its own: below about 40 positions per resident warp the streaming sweep is
+// bound by its serial chain (one 64^3 event: 27 us a sweep, tiled 8.4), and up
+// to eight events the launches cost less than that.
+constexpr long long kTilePositions = 40;
+constexpr int kTileEvents = 8;
+
+bool wants_tiles(const shasta_batch* b) {
+  if (b->tiles_off || b->force_range >= 0 || b->nlive > kTileEvents) return false;
+  for (int a = 0; a < 3; ++a)
+    if (total_positions(b, a) >= kTilePositions * warp_slots(b, 0, a, 0)) return false;
+  return true;
+}
+
+TilePlan tile_of(const shasta_batch* b, const Event& e, int axis) {
+  TilePlan t;
+  const int n = extent(e.g, axis);
+  t.shape = tile_shape_for(n, axis);
+  t.blocks_per_sm = b->tile_bps[e.eos.kind][axis][t.shape];
+  tile_cut(t, n);
+  return t;
+}
+
+// Readies the tiled kernels of all live events (before any capture).
+cudaError_t prepare_tiles(shasta_batch* b) {
+  for (const Event& e : b->ev) {
+    if (!e.live) continue;
+    const bool bag = e.eos.kind == SHASTA_EOS_BAG;
+    for (int a = 0; a < 3; ++a) {
+      const int shape = tile_shape_for(extent(e.g, a), a);
+      int& bps = b->tile_bps[e.eos.kind][a][shape];
+      if (bps) continue;
+      const cudaError_t ce =
+          b->mixed ? (bag ? prepare_tile_mixed_bag : prepare_tile_mixed_ideal)(a, shape, &bps)
+                   : (bag ? prepare_tile_f32_bag : prepare_tile_f32_ideal)(a, shape, &bps);
+      if (ce != cudaSuccess) return ce;
+    }
+  }
+  return cudaSuccess;
+}
+
 void drop_graph(shasta_batch* b) {
   if (b->graph) cudaGraphExecDestroy(b->graph);
   b->graph = nullptr;
@@ -349,7 +418,10 @@ shasta_status build_plan(shasta_batch* b) {
         for (int k = 0; k < 2; ++k)
           if (!groups[a][k].empty())
             b->plan[r][s].push_back(make_list(b, groups[a][k], a, k, host));
+      fit_ranges(b, b->plan[r][s], b->tune_var, b->tune_share);
     }
+  b->by_event = wants_tiles(b);
+  if (b->by_event) CK(prepare_tiles(b), "prepare tiled kernels");
   shasta_status st = upload_lists(b, host);
   if (st != SHASTA_OK) return st;
   b->plan_base = b->bsteps;
@@ -382,40 +454,104 @@ SweepParams batch_params(const shasta_batch* b, const LaunchRec& L, int from, in
   return P;
 }
 
-cudaError_t launch_rec(shasta_batch* b, const LaunchRec& L, int from, int variant,
-                       long long range, cudaStream_t st = nullptr) {
+cudaError_t launch_rec(shasta_batch* b, const LaunchRec& L, int from, cudaStream_t st) {
   if (!L.nlist || !L.items) return cudaSuccess;
-  if (!st) st = b->stream;
   ++b->launches;
-  const SweepParams P = batch_params(b, L, from, variant, range);
+  const SweepParams P = batch_params(b, L, from, L.variant, L.range);
   BatchList BL;
   BL.ev = b->d_desc;
   BL.idx = b->d_plan + L.idx_off;
-  BL.prefix = b->d_plan + (range < 1 ? L.gpre_off : L.pre_off);
+  BL.prefix = b->d_plan + (L.range < 1 ? L.gpre_off : L.pre_off);
   BL.nlist = L.nlist;
   return b->mixed ? launch_batch_mixed(P, BL, L.axis, L.eos, st)
                   : launch_batch_f32(P, BL, L.axis, L.eos, st);
 }
 
-// One step from plan index r: three sweep slots, each flipping the buffers.
-cudaError_t launch_step(shasta_batch* b, int r) {
+// Runs body(i, stream) for i < n with the streams side by side: 0 on the batch
+// stream, the others on side streams in turn, ordered after the batch stream's
+// earlier work and before its later work.
+template <class Body>
+cudaError_t side_by_side(shasta_batch* b, int n, Body body) {
+  const int nside = std::min(n - 1, shasta_batch::kSide);
+  cudaError_t e = cudaSuccess;
+  if (nside > 0) {
+    e = cudaEventRecord(b->fork, b->stream);
+    for (int i = 0; i < nside && e == cudaSuccess; ++i) e = cudaStreamWaitEvent(b->side[i], b->fork, 0);
+  }
+  for (int i = 0; i < n && e == cudaSuccess; ++i) {
+    const int k = i % (nside + 1);
+    e = body(i, k ? b->side[k - 1] : b->stream);
+  }
+  for (int i = 0; i < nside && e == cudaSuccess; ++i) {
+    e = cudaEventRecord(b->join[i], b->side[i]);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(b->stream, b->join[i], 0);
+  }
+  return e;
+}
+
+cudaError_t launch_slot(shasta_batch* b, const std::vector<LaunchRec>& V, int from) {
+  return side_by_side(b, (int)V.size(), [&](int i, cudaStream_t st) { return launch_rec(b, V[i], from, st); });
+}
+
+// One sweep of event i alone, tiled.
+cudaError_t launch_event(shasta_batch* b, int i, int axis, int from, bool chain, cudaStream_t st) {
+  const Event& e = b->ev[i];
+  const long long nx = e.g.nx, ny = e.g.ny;
+  SweepParams P;
+  memset(&P, 0, sizeof P);
+  P.qin = b->quad[from] + 4 * e.off;
+  P.rin = b->rf[from] + e.off;
+  P.qout = b->quad[from ^ 1] + 4 * e.off;
+  P.rout = b->rf[from ^ 1] + e.off;
+  P.n = extent(e.g, axis);
+  P.plane = plane_of(e.g, axis);
+  P.stride = axis == 0 ? 1 : (axis == 1 ? nx : nx * ny);
+  P.nb = axis == 0 ? (int)ny : (int)nx;
+  P.sb = axis == 0 ? nx : 1;
+  P.sc = axis == 2 ? nx : nx * ny;
+  P.bc = e.g.bc;
+  P.frozen = e.frozen ? (const float*)e.frozen + frozen_axis_offset(e.g.nx, e.g.ny, e.g.nz, axis) : nullptr;
+  P.tau_h = 0.5 * e.lambda;
+  P.tau_f = e.lambda;
+  P.htau_h = 0.5 * P.tau_h;
+  P.htau_f = 0.5 * P.tau_f;
+  P.eta = b->o.eta;
+  P.omd = 1.0 - b->o.delta;
+  P.bag_B = e.eos.B;
+  P.bag_ec = e.eos.e_c;
+  P.clamp_count = b->d_count + i;
+  set_float_scalars(P);
+  P.ncap = e.ncell;
+  P.chk = b->d_chk;
+  ++b->launches;
+  const TilePlan t = tile_of(b, e, axis);
+  const bool bag = e.eos.kind == SHASTA_EOS_BAG;
+  return b->mixed ? (bag ? launch_tile_mixed_bag : launch_tile_mixed_ideal)(P, t, axis, b->sm_count, chain, st)
+                  : (bag ? launch_tile_f32_bag : launch_tile_f32_ideal)(P, t, axis, b->sm_count, chain, st);
+}
+
+// One step from plan index r (ahead: steps queued in the same call whose
+// counts are not booked yet; single: not inside a graph): three sweep slots,
+// each flipping the buffers.  Events on launches of their own do not wait for
+// one another within a step.
+cudaError_t launch_step(shasta_batch* b, int r, int ahead, bool single) {
+  if (b->by_event) {
+    std::vector<int> ids;
+    for (int i = 0; i < (int)b->ev.size() && (int)ids.size() < b->nlive; ++i)
+      if (b->ev[i].live) ids.push_back(i);
+    const int cur = b->cur;
+    const cudaError_t e = side_by_side(b, (int)ids.size(), [&](int j, cudaStream_t st) {
+      const int ph = (int)((b->ev[ids[j]].steps + ahead) % 6);
+      cudaError_t ce = cudaSuccess;
+      for (int s = 0; s < 3 && ce == cudaSuccess; ++s)
+        ce = launch_event(b, ids[j], kAxisTable[3 * ph + s], cur ^ (s & 1), single && ids.size() == 1, st);
+      return ce;
+    });
+    b->cur ^= 1;
+    return e;
+  }
   for (int s = 0; s < 3; ++s) {
-    const std::vector<LaunchRec>& V = b->plan[r][s];
-    const int nside = std::min((int)V.size() - 1, shasta_batch::kSide);
-    cudaError_t e = cudaSuccess;
-    if (nside > 0) {
-      e = cudaEventRecord(b->fork, b->stream);
-      for (int i = 0; i < nside && e == cudaSuccess; ++i) e = cudaStreamWaitEvent(b->side[i], b->fork, 0);
-    }
-    for (size_t i = 0; i < V.size() && e == cudaSuccess; ++i) {
-      const int k = (int)i - 1;  // launch 0 on the batch stream, the others on side streams
-      cudaStream_t st = k >= 0 && k < nside ? b->side[k] : b->stream;
-      e = launch_rec(b, V[i], b->cur, b->tune_var[V[i].axis], b->tune_range[V[i].axis], st);
-    }
-    for (int i = 0; i < nside && e == cudaSuccess; ++i) {
-      e = cudaEventRecord(b->join[i], b->side[i]);
-      if (e == cudaSuccess) e = cudaStreamWaitEvent(b->stream, b->join[i], 0);
-    }
+    const cudaError_t e = launch_slot(b, b->plan[r][s], b->cur);
     if (e != cudaSuccess) return e;
     b->cur ^= 1;
   }
@@ -443,32 +579,27 @@ shasta_status autotune(shasta_batch* b) {
         if (b->ev[i].live && b->ev[i].eos.kind == k) ids.push_back(i);
       if (!ids.empty()) recs.push_back(make_list(b, ids, a, k, host));
     }
+    b->trial = true;
     st = upload_lists(b, host);
+    b->trial = false;
     if (st != SHASTA_OK) break;
-    const long long total = total_positions(b, a);
     float best = 1e30f;
     int bv = 0;
-    long long br = b->tune_range[a];
-    double bsh = 0.0;
+    double bsh = b->tune_share[a];
     // one sweep of every event per choice after an untimed one, five where
     // that is short (two runs of a choice differ by 0.1% at 0.1 ms and more);
     // the other register variant for the best share only.  Every trial is
     // time taken from the batch's own steps: 32 sweeps an axis were a third
     // of a 48-step batch, these are 10.
-    auto sweep_all = [&](int var, long long range) {
-      cudaError_t ce = cudaSuccess;
-      for (const LaunchRec& L : recs)
-        if (ce == cudaSuccess) ce = launch_rec(b, L, b->cur, var, range);
-      return ce;
-    };
     auto trial = [&](int var, double sh) {
-      // share 0: whole line groups
-      const long long range = sh > 0 ? range_for(total, warp_slots(b, 0, a, var), sh) : 0;
-      cudaError_t ce = sweep_all(var, range);
+      const int vars[3] = {var, var, var};
+      const double shs[3] = {sh, sh, sh};
+      fit_ranges(b, recs, vars, shs);
+      cudaError_t ce = launch_slot(b, recs, b->cur);
       float ms = 0;
       for (int reps = 1; reps <= 5 && ce == cudaSuccess; reps += 4) {
         ce = cudaEventRecord(e0, b->stream);
-        for (int r = 0; r < reps && ce == cudaSuccess; ++r) ce = sweep_all(var, range);
+        for (int r = 0; r < reps && ce == cudaSuccess; ++r) ce = launch_slot(b, recs, b->cur);
         if (ce == cudaSuccess) ce = cudaEventRecord(e1, b->stream);
         if (ce == cudaSuccess) ce = cudaEventSynchronize(e1);
         if (ce == cudaSuccess) ce = cudaEventElapsedTime(&ms, e0, e1);
@@ -480,7 +611,6 @@ shasta_status autotune(shasta_batch* b) {
       } else if (ms < best) {
         best = ms;
         bv = var;
-        br = range;
         bsh = sh;
       }
     };
@@ -488,7 +618,7 @@ shasta_status autotune(shasta_batch* b) {
       if (st == SHASTA_OK) trial(0, sh);
     if (st == SHASTA_OK) trial(1, bsh);
     b->tune_var[a] = bv;
-    b->tune_range[a] = br;
+    b->tune_share[a] = bsh;
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
@@ -596,6 +726,8 @@ shasta_status shasta_batch_create(const shasta_batch_opts* o, shasta_batch** out
       b->sm_count = sms;
     const char* v = getenv("SHASTA_BATCH_RANGE");
     if (v && atoll(v) >= 0) b->force_range = atoll(v);
+    v = getenv("SHASTA_TILE");
+    if (v && !strcmp(v, "off")) b->tiles_off = true;
   }
   auto bail = [&](cudaError_t err, const char* where) {
     std::string m = std::string(where) + ": " + cudaGetErrorString(err);
@@ -797,6 +929,8 @@ shasta_status batch_add_enqueue(shasta_batch* b, const shasta_grid* g, double dx
 
 shasta_status batch_remove_enqueue(shasta_batch* b, int id) { return remove_impl(b, id, false); }
 
+void batch_share_launches(shasta_batch* b) { b->tiles_off = true; }
+
 shasta_status batch_extract_enqueue(shasta_batch* b, int id, double* const prims[6],
                                     double* const cons[5], unsigned long long* counter) {
   Event* e = find(b, id);
@@ -835,12 +969,10 @@ shasta_status shasta_batch_step(shasta_batch* b, int nsteps) {
   DeviceGuard dg(b->device);
   if (!b->tuned) {
     model_choice(b);
-    if (b->o.autotune && b->force_range < 0) {
+    if (b->o.autotune && b->force_range < 0 && !wants_tiles(b)) {
       shasta_status st = autotune(b);
       if (st != SHASTA_OK) return st;
     }
-    if (b->force_range >= 0)
-      for (int a = 0; a < 3; ++a) b->tune_range[a] = b->force_range;
     b->tuned = true;
     b->plan_valid = false;
   }
@@ -861,7 +993,7 @@ shasta_status shasta_batch_step(shasta_batch* b, int nsteps) {
         cudaGraph_t gr = nullptr;
         CK(cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal), "begin capture");
         cudaError_t ce = cudaSuccess;
-        for (int k = 0; k < 6 && ce == cudaSuccess; ++k) ce = launch_step(b, (r + k) % 6);
+        for (int k = 0; k < 6 && ce == cudaSuccess; ++k) ce = launch_step(b, (r + k) % 6, k, false);
         cudaError_t ce2 = cudaStreamEndCapture(b->stream, &gr);
         b->cur = cur0;
         b->graph_launches = b->launches - l0;
@@ -883,7 +1015,7 @@ shasta_status shasta_batch_step(shasta_batch* b, int nsteps) {
       b->launches += b->graph_launches;
       done = 6;  // 18 buffer flips: cur unchanged
     } else {
-      CK(launch_step(b, r), "batched sweep launch");
+      CK(launch_step(b, r, 0, true), "batched sweep launch");
     }
     b->bsteps += done;
     for (int i = 0; i < n; ++i)
@@ -1031,6 +1163,7 @@ shasta_status shasta_batch_info(shasta_batch* b, int64_t out[7]) {
         ++launches;
         items += L.items;
       }
+    if (b->by_event) launches = 3 * b->nlive;
   }
   out[4] = launches;
   out[5] = items;

@@ -24,4 +24,8 @@ shasta_status batch_remove_enqueue(shasta_batch* b, int id);
 shasta_status batch_extract_enqueue(shasta_batch* b, int id, double* const prims[6],
                                     double* const cons[5], unsigned long long* counter);
 
+// Keeps every sweep of the batch in launches shared by its events (the serving
+// loop counts on at most one launch per EoS and sweep slot, whatever the mix).
+void batch_share_launches(shasta_batch* b);
+
 }  // namespace shasta

@@ -659,6 +659,7 @@ shasta_status shasta_server_create(const shasta_server_opts* o, shasta_server** 
   bo.capacity_cells = std::min<long long>(cells, 1LL << 31);
   shasta_status st = shasta_batch_create(&bo, &s->batch);
   if (st != SHASTA_OK) return bail(st, std::string("batch: ") + shasta_batch_last_error(nullptr));
+  shasta::batch_share_launches(s->batch);
   s->pool_cells = bo.capacity_cells;
   s->worker = std::thread(worker_main, s);
   s->deliverer = std::thread(deliverer_main, s);

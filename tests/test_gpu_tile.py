@@ -60,3 +60,38 @@ def test_small_grids_take_tiles(monkeypatch, shape):
     assert all(r <= n for r, n in zip(got[2], shape))
     for a, b in zip(ref[0], got[0]):
         assert np.array_equal(a, b)
+
+
+BATCH = [((40, 36, 28), "reflect", "ideal"), ((33, 20, 48), "periodic", "bag"), ((24, 40, 16), "frozen", "ideal"),
+         ((64, 64, 64), "reflect", "bag"), ((5, 3, 2), "reflect", "ideal"), ((1, 33, 1), "frozen", "bag"),
+         ((48, 48, 48), "reflect", "ideal"), ((17, 9, 30), "periodic", "ideal"), ((70, 31, 9), "reflect", "bag")]
+
+
+@pytest.mark.parametrize("precision", ["fp32", "mixed"])
+@pytest.mark.parametrize("count", [1, 2, 7, 8, 9])
+def test_small_batches_by_event_match_streaming_bitwise(monkeypatch, precision, count):
+    """Up to eight small events take tiled launches of their own, more the
+    shared streaming launches: the same states and clamp counts, with events at
+    different phases, through graphs and single steps, and after a removal."""
+    require_gpu()
+    res = []
+    for tile in ("off", ""):
+        monkeypatch.setenv("SHASTA_TILE", tile)
+        with S.Batch(600_000, precision=precision, check_input=False) as b:
+            ids = []
+            for i, (shape, bc, eos) in enumerate(BATCH[:count]):
+                pr = W.random_state(shape, seed=40 + i, vmax=0.6, e_range=(0.3, 3.0))
+                U = oracle().prim2cons(OR.params(shape), *pr.as_list())
+                U[1].flat[-1] = 1.5 * U[0].flat[-1]
+                ids.append(b.add_conserved(shape, U, bc=bc, eos=eos))
+                if i == 1:
+                    b.step(2)
+            b.step(7)
+            if count > 2:
+                b.remove(ids.pop(1))
+            b.step(8)
+            res.append([(b.get_conserved(e), b.counters(e), b.steps_done(e)) for e in ids])
+    for (ua, ca, sa), (ub, cb, sb) in zip(*res):
+        assert sa == sb and ca == cb > 0
+        for x, y in zip(ua, ub):
+            assert np.array_equal(x, y)
