@@ -3,7 +3,9 @@
 // footprint, advances them together and hands finished results back.
 #include <cuda_runtime.h>
 #include <math.h>
+#include <stdlib.h>
 #include <string.h>
+#include <sys/mman.h>
 
 #include <algorithm>
 #include <chrono>
@@ -39,11 +41,39 @@ constexpr size_t kBounceHalf = 16u << 20; // bytes per half of a pinned bounce b
 
 enum JobState { J_WAIT, J_STAGED, J_RESIDENT, J_OUT, J_DONE, J_FAILED };
 
+// Uninitialised host memory for an event's inputs.  Large ones come on 2 MB
+// boundaries with huge pages asked for: the copy into fresh memory is bound by
+// its first-touch faults.
+struct HostBuf {
+  double* p = nullptr;
+  HostBuf() = default;
+  HostBuf(const HostBuf&) = delete;
+  HostBuf& operator=(const HostBuf&) = delete;
+  ~HostBuf() { release(); }
+  bool allocate(size_t bytes) {
+    constexpr size_t kHuge = 2u << 20;
+    void* q = nullptr;
+    if (bytes < 2 * kHuge) {
+      q = malloc(bytes);
+    } else if (posix_memalign(&q, kHuge, (bytes + kHuge - 1) / kHuge * kHuge) != 0) {
+      q = nullptr;
+    } else {
+      madvise(q, (bytes + kHuge - 1) / kHuge * kHuge, MADV_HUGEPAGE);  // (a wish: its failure costs time only)
+    }
+    p = static_cast<double*>(q);
+    return p != nullptr;
+  }
+  void release() {
+    free(p);
+    p = nullptr;
+  }
+};
+
 struct Job {
   uint64_t ticket = 0;
   shasta_event ev{};
   long long ncell = 0;
-  std::vector<double> in;  // the five input arrays, copied at submit
+  HostBuf in;  // the five input arrays, copied at submit
   JobState st = J_WAIT;
   shasta_status status = SHASTA_OK;
   double t_submit = 0, t_admit = 0, t_done = 0;
@@ -342,7 +372,7 @@ void release_input(shasta_server* s, const JobP& j) {
   j->chk = -1;
   if (j->in_off >= 0) s->in_arena.release(j->in_off, 5 * j->ncell * (long long)sizeof(double));
   j->in_off = -1;
-  std::vector<double>().swap(j->in);
+  j->in.release();
 }
 
 // Copies the next queue heads into input staging on the copy stream (first
@@ -384,7 +414,7 @@ bool stage(shasta_server* s) {
     for (int k = 0; k < 5; ++k) f[k] = d + (size_t)k * j->ncell;
     cudaError_t e = cudaEventCreateWithFlags(&j->in_ready, cudaEventDisableTiming);
     if (e == cudaSuccess)
-      e = cudaMemcpyAsync(d, j->in.data(), 5 * j->ncell * sizeof(double), cudaMemcpyHostToDevice,
+      e = cudaMemcpyAsync(d, j->in.p, 5 * j->ncell * sizeof(double), cudaMemcpyHostToDevice,
                           s->copy);
     if (e == cudaSuccess)
       e = launch_check(j->ev.kind == SHASTA_STATE_PRIMITIVE, f, (size_t)j->ncell, s->d_chk + 2 * c, s->h_chk + c,
@@ -711,13 +741,16 @@ shasta_status shasta_submit(shasta_server* s, const shasta_event* ev, uint64_t* 
   j->ev = *ev;
   for (int k = 0; k < 5; ++k) j->ev.fields[k] = nullptr;
   j->ncell = ncell;
-  try {
-    j->in.resize(5 * (size_t)ncell);
-  } catch (const std::bad_alloc&) {
-    return fail(s, SHASTA_ENOMEM, "host copy of the input");
+  if (!j->in.allocate(5 * (size_t)ncell * sizeof(double))) return fail(s, SHASTA_ENOMEM, "host copy of the input");
+  for (int k = 0; k < 5; ++k) {
+    char* dst = (char*)(j->in.p + (size_t)k * ncell);
+    const size_t len = (size_t)ncell * sizeof(double);
+    // threads from 4 MB a field on (starting them takes about 0.1 ms)
+    if (len >= (4u << 20))
+      par_copy(dst, (const char*)ev->fields[k], len);
+    else
+      memcpy(dst, ev->fields[k], len);
   }
-  for (int k = 0; k < 5; ++k)
-    memcpy(j->in.data() + (size_t)k * ncell, ev->fields[k], ncell * sizeof(double));
   {
     std::lock_guard<std::mutex> lk(s->mu);
     if (s->fatal != SHASTA_OK) return SHASTA_ECUDA;
