@@ -46,6 +46,8 @@ Kern kern_of(int i) {
     case 6: return kern<EOS, REC, AXIS, 6>();
     case 7: return kern<EOS, REC, AXIS, 7>();
     case 8: return kern<EOS, REC, AXIS, 8>();
+    case 9: return kern<EOS, REC, AXIS, 9>();
+    case 10: return kern<EOS, REC, AXIS, 10>();
   }
   return Kern{nullptr, 0, 0, 0};
 }

@@ -15,7 +15,7 @@ from gpu_util import oracle, require_gpu
 
 pytestmark = pytest.mark.gpu
 
-OWN = [52, 68, 84, 100, 116, 132, 148, 180, 212]  # own positions of each tile shape
+OWN = [52, 68, 84, 100, 116, 132, 148, 180, 212, 244, 276]  # own positions of each tile shape
 TABLE = np.arange(4001) * 0.01 / 3.0
 
 
