@@ -860,15 +860,19 @@ shasta_status shasta_create(const shasta_grid* g, double dx, double lambda, cons
   if (e.kind == SHASTA_EOS_TABLE) {
     const size_t n = (size_t)e.table_n;
     const size_t b64 = ((n * sizeof(double) + 255) / 256) * 256;
-    err = cudaMalloc(&c->tab_mem, b64 + n * sizeof(float));
+    err = cudaMalloc(&c->tab_mem, b64 + n * sizeof(float2));
     if (err != cudaSuccess) return bail(err, "cudaMalloc EoS table");
-    std::vector<float> t32(e.table, e.table + n);
+    std::vector<float2> t32(n);
+    for (size_t k = 0; k < n; ++k) {
+      const float a = (float)e.table[k];
+      t32[k] = make_float2(a, k + 1 < n ? (float)e.table[k + 1] - a : 0.0f);
+    }
     err = cudaMemcpy(c->tab_mem, e.table, n * sizeof(double), cudaMemcpyHostToDevice);
     if (err == cudaSuccess)
-      err = cudaMemcpy((char*)c->tab_mem + b64, t32.data(), n * sizeof(float), cudaMemcpyHostToDevice);
+      err = cudaMemcpy((char*)c->tab_mem + b64, t32.data(), n * sizeof(float2), cudaMemcpyHostToDevice);
     if (err != cudaSuccess) return bail(err, "copy EoS table");
     c->tab.p64 = (const double*)c->tab_mem;
-    c->tab.p32 = (const float*)((char*)c->tab_mem + b64);
+    c->tab.p32 = (const float2*)((char*)c->tab_mem + b64);
     c->tab.n = e.table_n;
     c->tab.de = e.table_de;
     c->tab.inv_de32 = (float)(1.0 / e.table_de);

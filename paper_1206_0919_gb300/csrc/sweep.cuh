@@ -34,6 +34,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "eos_table.cuh"
+
 namespace shasta {
 
 constexpr int NF = 5;  // E, M_x, M_y, M_z, R
@@ -41,17 +43,6 @@ constexpr int NG = 3;  // ghost depth of one SHASTA pass
 
 enum { BC_REFLECT = 0, BC_PERIODIC = 1, BC_FROZEN = 2 };
 enum { EOS_IDEAL = 0, EOS_BAG = 1, EOS_TABLE = 2 };
-
-// Tabulated EoS (EOS_TABLE): p at e = k de, k = 0 .. n-1, linear in
-// between, the last interval continued above the table (device copies in
-// double and float).
-struct EosTable {
-  const double* p64;
-  const float* p32;
-  int n;
-  double de;
-  float inv_de32;  // 1 / de in float (FP32 lookups)
-};
 
 // Geometry and constants of one sweep launch (filled on the host).
 struct SweepParams {

@@ -281,43 +281,6 @@ __device__ __forceinline__ void copy_cell(const SweepParams& P, const Geo& G, fl
 
 // ----------------------------------------------------------- recovery ----
 
-// p(e) of a tabulated EoS in float: linear between the nodes k de, the
-// last interval continued above (the index stays inside the table for any
-// e, NaN included); *slope receives dp/de of the interval.
-__device__ __forceinline__ float tab32(const EosTable& T, float e, float* slope = nullptr) {
-  const float x = e * T.inv_de32;
-  int k = (int)x;
-  k = k < 0 ? 0 : (k > T.n - 2 ? T.n - 2 : k);
-  const float f = x - (float)k;
-  const float a = __ldg(T.p32 + k), b = __ldg(T.p32 + k + 1);
-  if (slope) *slope = (b - a) * T.inv_de32;
-  return fmaf(f, b - a, a);
-}
-
-// Tabulated EoS: p from E and |M|^2.  The root is the fixed point of Sec. 3,
-// |v| = |M| / (E + p(E - |M| |v|)), started as there from |M| / (E + p(E)).
-// In float the root is found by Newton steps on g(v) = v - |M| / (E + p),
-// g'(v) = 1 - |M|^2 p'(e) / (E + p)^2 >= 1 - v^2 p' > 0 (exact within one
-// interval of the piecewise-linear table), until the change is at most
-// 1e-7 (12 steps at most), then p = p(E - |M| |v|).
-__device__ __forceinline__ float table_p32(const EosTable& T, float E, float M2) {
-  const float M = sqrtf(M2);
-  float v = M * __fdividef(1.0f, E + tab32(T, E));
-#pragma unroll 1
-  for (int it = 0; it < 12; ++it) {
-    float dp;
-    const float pe = tab32(T, fmaf(-M, v, E), &dp);
-    const float r = __fdividef(1.0f, E + pe);
-    const float g = fmaf(-M, r, v);               // v - M / (E + p)
-    const float mr = M * r;
-    const float gp = fmaf(-mr * mr, dp, 1.0f);    // 1 - M^2 p' / (E + p)^2
-    const float d = __fdividef(g, gp);
-    v -= d;
-    if (fabsf(d) <= 1e-7f) break;
-  }
-  return tab32(T, fmaf(-M, v, E));
-}
-
 // Recovery arithmetic of the kernels on a float state: REC_F32 all in
 // float (precision FP32); REC_DF |M|^2 and D = E^2 - |M|^2 in double-float,
 // the rest in float (MIXED); REC_F64 D, the root s, p and w in double from
@@ -412,6 +375,37 @@ __device__ __forceinline__ unsigned rec64(float Ef, float mxf, float myf, float 
   return rec64_rest<EOS>(Ef, mxf, myf, mzf, m1f, omd, B, ec, w, p);
 }
 
+// rec32 of N cells with a tabulated EoS in FP32, their roots taken together;
+// cl[i]: |M| was clamped or E <= 0.
+template <int N>
+__device__ __forceinline__ void rec32_table(const float (&E)[N], const float (&mx)[N], const float (&my)[N],
+                                            const float (&mz)[N], const float (&m1)[N], float omd,
+                                            const EosTable& T, float (&w)[N], float (&p)[N], bool (&cl)[N]) {
+  float M2[N], m[N];
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    M2[i] = fmaf(mx[i], mx[i], fmaf(my[i], my[i], mz[i] * mz[i]));
+    const float lim = omd * E[i];
+    const float L2 = lim * lim;
+    m[i] = m1[i];
+    cl[i] = M2[i] > L2;
+    if (cl[i]) {
+      m[i] = m1[i] * (lim * rsqrtf(M2[i]));
+      M2[i] = L2;
+    }
+  }
+  table_p32<N>(T, E, M2, p);
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    w[i] = m[i] * __fdividef(1.0f, E[i] + p[i]);
+    if (!(E[i] > 0.0f)) {
+      w[i] = 0.0f;
+      p[i] = 0.0f;
+      cl[i] = true;
+    }
+  }
+}
+
 // Velocity along the sweep and pressure of one cell, FP32 (REC_DF: D in
 // double-float; REC_F64: rec64).  mx, my, mz are the momenta, m1 the one
 // along the sweep.  Returns 1 if |M| was clamped or E <= 0.
@@ -421,6 +415,14 @@ __device__ __forceinline__ unsigned rec32(float E, float mx, float my, float mz,
                                           const EosTable& T, float& w, float& p) {
   if constexpr (REC == REC_F64 && EOS != EOS_TABLE)
     return rec64<EOS>(E, mx, my, mz, m1, omd64, B, ec, w, p);
+  if constexpr (EOS == EOS_TABLE) {
+    float wa[1], pa[1];
+    bool cl[1];
+    rec32_table<1>({E}, {mx}, {my}, {mz}, {m1}, omd, T, wa, pa, cl);
+    w = wa[0];
+    p = pa[0];
+    return cl[0] ? 1u : 0u;
+  }
   unsigned clamped = 0;
   float M2, M2lo = 0.0f;  // |M|^2; REC_DF: an unevaluated sum M2 + M2lo
   if constexpr (REC == REC_DF) {
@@ -457,9 +459,7 @@ __device__ __forceinline__ unsigned rec32(float E, float mx, float my, float mz,
     D = E2 - M2;
   }
   float pp;
-  if constexpr (EOS == EOS_TABLE) {
-    pp = table_p32(T, E, M2);
-  } else if constexpr (EOS == EOS_BAG) {
+  if constexpr (EOS == EOS_BAG) {
     // One root for both branches.  With R0 = E^2 + 3D the ideal-gas root
     // e = sqrt(R0) - E lies above e_c exactly when R0 > (E + e_c)^2; then
     // the bag root with p = (e - 4b)/3, else b = 0, which is the ideal-gas
@@ -501,6 +501,15 @@ template <int EOS, int REC>
 __device__ __forceinline__ void rec2(f2 E, f2 mx, f2 my, f2 mz, f2 mpar, float omd, double omd64,
                                      float B, float ec, const EosTable& T, f2& w, f2& p,
                                      unsigned& cnt, bool in_seg) {
+  if constexpr (EOS == EOS_TABLE) {
+    float wa[2], pa[2];
+    bool cl[2];
+    rec32_table<2>({E.x, E.y}, {mx.x, mx.y}, {my.x, my.y}, {mz.x, mz.y}, {mpar.x, mpar.y}, omd, T, wa, pa, cl);
+    if (cl[0]) cnt += in_seg ? 1u : 0u;
+    w = f2{wa[0], wa[1]};
+    p = f2{pa[0], pa[1]};
+    return;
+  }
   float wl, wh, pl, ph;
   const unsigned c =
       rec32<EOS, REC>(E.x, mx.x, my.x, mz.x, mpar.x, omd, omd64, B, ec, T, wl, pl);

@@ -457,7 +457,17 @@ __global__ void __launch_bounds__(Lay<AXIS, C, XL>::WARPS * 32, MINB)
 #pragma unroll 1
     for (int h = 0; h < 2; ++h) {
       float w[C + 2], p[C + 2];
-      if constexpr (EOS == EOS_TABLE || REC == fast::REC_F64) {
+      if constexpr (EOS == EOS_TABLE) {
+        float wc[C], pc[C];
+        bool cl[C];
+        fast::rec32_table<C>(H[0], H[1], H[2], H[3], H[1 + AXIS], P.f_omd, P.tab, wc, pc, cl);
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+          w[c + 1] = wc[c];
+          p[c + 1] = pc[c];
+          if (cl[c] && h == 0) nclamp += valid && (unsigned)(pos0 + c - s0) < (unsigned)(s1 - s0) ? 1u : 0u;
+        }
+      } else if constexpr (REC == fast::REC_F64) {
 #pragma unroll
         for (int c = 0; c < C; ++c) {
           const unsigned cl = fast::rec32<EOS, REC>(H[0][c], H[1][c], H[2][c], H[3][c], H[1 + AXIS][c], P.f_omd,
