@@ -114,3 +114,51 @@ def test_primitive_maps_against_oracle(eos, scale):
         got, ref = s.get_primitives(), O.recover(P, U)
         for k in ("e", "vx", "vy", "vz", "n", "p"):
             assert max_rel_err(got[k], ref[k]) <= 1e-13, k
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("name,slopes", [("ideal", [1 / 3]), ("kinked", [0.6, 0.0]), ("two values", [0.2])])
+def test_table_primitives_against_extended_precision(name, slopes, precision):
+    """The root M = (E + p(E - M v)) v of the tabulated EoS against a plain
+    fixed point in extended precision: cells at rest, |v| from 1e-30 to 1 - 1e-9,
+    energies below, in and above the table, and some (1e-25, 1e35) that leave
+    the range of the float steps.  A last change of at most 1e-14 leaves
+    1e-14 c / (1 - c) at a contraction c <= max p', and four roundings."""
+    require_gpu()
+    de, shape = 0.01, (50, 20, 4)
+    nodes = 2 if name == "two values" else 1001
+    table = np.concatenate([[0.0], np.cumsum(np.resize(slopes, nodes - 1) * de)])
+    rng = np.random.default_rng(5)
+    n = 4000
+    E = 10.0 ** rng.uniform(-4, 2, n)
+    frac = np.where(rng.random(n) < 0.5, rng.uniform(0, 1, n), 1 - 10.0 ** rng.uniform(-9, -1, n))
+    frac[:200] = 10.0 ** rng.uniform(-30, -1, 200)
+    frac[200:300] = 0.0
+    if precision == "fp64":
+        E[300:400], E[400:500] = 1e-25, 1e35
+    M = E * frac
+    if precision == "fp32":
+        frac = np.minimum(frac, 1 - 1e-5)
+        E = E.astype(np.float32).astype(np.float64)
+        M = (E * frac).astype(np.float32).astype(np.float64)
+    zero = np.zeros(n)
+    with S.Solver(shape, precision=precision, check_input=False, autotune=False, eos="table", table=table,
+                  table_de=de) as s:
+        s.set_conserved([x.reshape(shape[::-1]) for x in (E, zero, M, zero, E)])
+        got = s.get_primitives()
+    T, h = table.astype(np.longdouble), np.longdouble(de)
+    El, Ml = E.astype(np.longdouble), M.astype(np.longdouble)
+
+    def p(e):
+        k = np.clip(np.floor(e / h), 0, nodes - 2).astype(int)
+        return T[k] + (e / h - k) * (T[k + 1] - T[k])
+
+    v = Ml / (El + p(El))
+    for _ in range(400):
+        v = Ml / (El + p(El - Ml * v))
+    c = max(slopes)
+    tol = (1e-14 * c + 4 * 2.0 ** -52) / (1 - c)
+    assert np.max(np.abs(got["vy"].ravel() - v)) <= tol
+    assert np.max(np.abs(got["e"].ravel() - (El - Ml * v)) / El) <= tol
+    assert np.max(np.abs(got["p"].ravel() - p(El - Ml * v)) / El) <= tol
+    assert not got["vx"].any() and not got["vz"].any()
