@@ -586,25 +586,27 @@ shasta_status autotune(shasta_batch* b) {
     float best = 1e30f;
     int bv = 0;
     double bsh = b->tune_share[a];
-    // one sweep of every event per choice after an untimed one, five where
-    // that is short (two runs of a choice differ by 0.1% at 0.1 ms and more);
-    // the other register variant for the best share only.  Every trial is
-    // time taken from the batch's own steps: 32 sweeps an axis were a third
-    // of a 48-step batch, these are 10.
+    // one sweep of every event per choice after an untimed one, three where
+    // that is short (the first choice tells; two runs of a choice differ by
+    // 0.1% at 0.1 ms and more); the other register variant for the best share
+    // only.  Every trial is time taken from the batch's own steps: 32 sweeps an
+    // axis were a third of a 48-step batch, these are 10, or 21 short ones.
+    int reps = 1;
     auto trial = [&](int var, double sh) {
       const int vars[3] = {var, var, var};
       const double shs[3] = {sh, sh, sh};
       fit_ranges(b, recs, vars, shs);
       cudaError_t ce = launch_slot(b, recs, b->cur);
       float ms = 0;
-      for (int reps = 1; reps <= 5 && ce == cudaSuccess; reps += 4) {
+      while (ce == cudaSuccess) {
         ce = cudaEventRecord(e0, b->stream);
         for (int r = 0; r < reps && ce == cudaSuccess; ++r) ce = launch_slot(b, recs, b->cur);
         if (ce == cudaSuccess) ce = cudaEventRecord(e1, b->stream);
         if (ce == cudaSuccess) ce = cudaEventSynchronize(e1);
         if (ce == cudaSuccess) ce = cudaEventElapsedTime(&ms, e0, e1);
         ms /= (float)reps;
-        if (ms > 0.2f) break;
+        if (reps > 1 || ms > 0.2f || best < 1e30f) break;
+        reps = 3;
       }
       if (ce != cudaSuccess) {
         st = cuda_fail(b, ce, "autotune");
