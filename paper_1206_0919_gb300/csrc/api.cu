@@ -361,8 +361,8 @@ SweepParams sweep_params(shasta_ctx* c, int axis, int from, int variant, long lo
   return P;
 }
 
-// FP64 kernel: one thread per line segment; default segment length for
-// about 1024 threads per SM, segments of at least 16 cells (each re-runs a
+// FP64 streaming kernel (lines that no block holds): one thread per line
+// segment; default segment length for about 1024 threads per SM, segments of at least 16 cells (each re-runs a
 // 6-cell halo per side).
 long long fp64_segment(const shasta_ctx* c, int axis) {
   const long long n = axis == 0 ? c->g.nx : (axis == 1 ? c->g.ny : c->g.nz);
@@ -438,8 +438,8 @@ cudaError_t launch_tile(shasta_ctx* c, int axis, const SweepParams& P) {
 }
 
 // Cuts the lines of an axis into tiles (FP64: into blocks of whole lines) and
-// readies the kernel; leaves the
-// axis to the streaming sweep where there is no tiled one.
+// readies the kernel; leaves the axis to the streaming sweep where there is no
+// tiled one.
 cudaError_t plan_tiles(shasta_ctx* c, int axis) {
   TilePlan& t = c->tile[axis];
   t.shape = -1;

@@ -22,6 +22,10 @@
 // ordered symmetrically (second difference as (d+ + d-) - 2d, flux
 // differences as A_j - A_{j-1}).
 //
+// FP64 contexts run it where a line does not fit a block's shared memory (over
+// 874 cells, under 3); elsewhere sweep_lines64.cuh has the same bits at 0.37 of
+// the double operations.
+//
 // Pipeline (q = position of the newest loaded cell, q = -6 .. n+5):
 //   U^n_q loaded, (w, p)^n_q recovered
 //   Uhat^h_{q-1}     transported half-step value
@@ -43,6 +47,18 @@ constexpr int NG = 3;  // ghost depth of one SHASTA pass
 
 enum { BC_REFLECT = 0, BC_PERIODIC = 1, BC_FROZEN = 2 };
 enum { EOS_IDEAL = 0, EOS_BAG = 1, EOS_TABLE = 2 };
+
+// Adds the lanes' counts of clamped cells to *count (null: not counted), one
+// atomic a warp.  Atomics on one address are served one after the other, about
+// two a nanosecond: with one a lane they were a tail on the sweeps of evolved
+// states (200^3 hot spots, step 120, 364,000 clamped cells a step: streamed x /
+// y / z 126 / 112 / 111 us, now 114 / 100 / 100; tiled x 124, now 106).
+__device__ __forceinline__ void add_clamps(unsigned long long* count, unsigned n) {
+  if (!count) return;
+  const unsigned m = __activemask();
+  n = __reduce_add_sync(m, n);
+  if (n && (int)(threadIdx.x & 31) == __ffs(m) - 1) atomicAdd(count, (unsigned long long)n);
+}
 
 // Geometry and constants of one sweep launch (filled on the host).
 struct SweepParams {
@@ -517,7 +533,7 @@ __global__ void __launch_bounds__(128) sweep_kernel(SweepParams P) {
       static_cast<T*>(P.out[4])[i] = outv[4];
     }
   }
-  if (nclamp && P.clamp_count) atomicAdd(P.clamp_count, (unsigned long long)nclamp);
+  add_clamps(P.clamp_count, nclamp);
 }
 
 }  // namespace shasta

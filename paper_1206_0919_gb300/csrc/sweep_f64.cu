@@ -1,6 +1,8 @@
-// sweep_f64.cu -- FP64 instances of the fused sweep.  Built with
-// -fmad=false and IEEE division / square root so that the arithmetic is the
-// plain double-precision evaluation of each expression in source order.
+// sweep_f64.cu -- FP64 instances of the fused sweep: whole lines in shared
+// memory (sweep_lines64.cuh), or one thread per line segment (sweep.cuh).
+// Built with -fmad=false and IEEE division / square root so that the
+// arithmetic is the plain double-precision evaluation of each expression in
+// source order.
 #include "kernels.h"
 #include "chain.cuh"
 #include "sweep_lines64.cuh"

@@ -4,6 +4,9 @@
 // recovery at n+1/2, full step from the old state), reorganised for
 // throughput on Blackwell:
 //
+// Large grids and batches run it; single contexts take sweep_tile.cuh (the
+// same bits) along x and on grids with too few positions per warp (api.cu).
+//
 //  * State layout: (E, Mx, My, Mz) as one 16-byte quad per cell and R as a
 //    separate array.  A cell moves with one 16-byte and one 4-byte access,
 //    and the quad splits into the register pairs (E, Mx), (My, Mz).
@@ -1065,7 +1068,7 @@ __device__ __forceinline__ void sweep_items(const SweepParams& P, const BatchLis
         const int k = entry(r);
         const GeoR G{geo_of<AXIS>(L.ev[L.idx[k]])};
         sweep_item<EOS, AXIS, REC, RING, DIST, AF>(P, G, r - L.prefix[k], 0, G.n(), wsm, lane, nclamp);
-        if (nclamp && G.g.clamp) atomicAdd(G.g.clamp, (unsigned long long)nclamp);
+        add_clamps(G.g.clamp, nclamp);
         nclamp = 0;
       }
       return;
@@ -1085,7 +1088,7 @@ __device__ __forceinline__ void sweep_items(const SweepParams& P, const BatchLis
         const int s0 = loc - g * n;
         const int pe = min(end, x - s0 + n);  // the piece ends with the range or the line group
         sweep_item<EOS, AXIS, REC, RING, DIST, AF>(P, G, g, s0, s0 + (pe - x), wsm, lane, nclamp);
-        if (nclamp && G.g.clamp) atomicAdd(G.g.clamp, (unsigned long long)nclamp);
+        add_clamps(G.g.clamp, nclamp);
         nclamp = 0;
         x = pe;
       }
@@ -1117,7 +1120,7 @@ __device__ __forceinline__ void sweep_items(const SweepParams& P, const BatchLis
         x = pe;
       }
     }
-    if (nclamp && P.clamp_count) atomicAdd(P.clamp_count, (unsigned long long)nclamp);
+    add_clamps(P.clamp_count, nclamp);
   }
 }
 

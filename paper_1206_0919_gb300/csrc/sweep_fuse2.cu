@@ -239,7 +239,7 @@ __global__ void __launch_bounds__(32, 8) fuse2_kernel(SweepParams P, Geo2 G) {
     }
     __syncwarp();
   }
-  if (nclamp && P.clamp_count) atomicAdd(P.clamp_count, (unsigned long long)nclamp);
+  add_clamps(P.clamp_count, nclamp);
 }
 
 template <int EOS, int AA, int AB>

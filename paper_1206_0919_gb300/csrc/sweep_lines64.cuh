@@ -305,7 +305,7 @@ __global__ void __launch_bounds__(kLinesMaxThreads) sweep_lines_kernel(SweepPara
     });
     if (h == 0) __syncthreads();
   }
-  if (nclamp && P.clamp_count) atomicAdd(P.clamp_count, (unsigned long long)nclamp);
+  add_clamps(P.clamp_count, nclamp);
 }
 
 }  // namespace lines64

@@ -583,7 +583,7 @@ __global__ void __launch_bounds__(Lay<AXIS, C, XL>::WARPS * 32, MINB)
     k = kn;
   }
   cp_wait<0>();
-  if (nclamp && P.clamp_count) atomicAdd(P.clamp_count, (unsigned long long)nclamp);
+  add_clamps(P.clamp_count, nclamp);
 }
 
 }  // namespace tile
