@@ -28,8 +28,8 @@
 //    body (recovery, transport factors, the passes of the field pairs), which
 //    keeps the unrolled code within the instruction cache (unrolled twice it
 //    measured 60% of the time lost to fetch stalls more).
-//  * The cells of a lane are recovered without branches; a lane that holds a
-//    clamped or a vacuum cell (rare) takes all its cells again by rec32.
+//  * The cells of a lane are recovered without branches, with the clamp and
+//    the vacuum rule in warps that hold such a cell only.
 //  * (E, Mx) and (My, Mz) go through packed f32x2 arithmetic: 241 instead of
 //    278 instructions per 32 cells, 103 instead of 109 us (200^3, y).
 //  * y/z: the four warps of a block copy a tile of 8 adjacent lines, so that
@@ -242,13 +242,15 @@ __device__ __forceinline__ void coeffs(float tau, const float (&w)[C + 2], float
   }
 }
 
-// fast::rec32 for a cell that is neither clamped nor vacuum, the same
-// operations; ok is cleared where it is one of the two (w and p then have to
-// be taken from rec32).
-template <int EOS, int REC>
-__device__ __forceinline__ void rec_plain(float E, float mx, float my, float mz, float m, float omd, float B,
-                                          float ec, float& w, float& p, bool& ok) {
-  float M2, M2lo = 0.0f;
+// rec32 (REC_F32, REC_DF) in two parts, so that the cells of a lane are
+// recovered without branches: |M|^2 of all of them, then the roots, with the
+// clamp and the vacuum rule as selections (CLAMP) only where a lane of the warp
+// holds such a cell.  Evolved states hold many (hot spots, 200^3, step 120:
+// 1.5% of the recoveries); recovering such a lane's cells again by rec32 took
+// 106 us along x there, this 101; 92 before the first clamp.
+template <int REC>
+__device__ __forceinline__ float norm2(float mx, float my, float mz, float& lo) {
+  lo = 0.0f;
   if constexpr (REC == fast::REC_DF) {
     const float a = mx * mx, a_l = fmaf(mx, mx, -a);
     const float b = my * my, b_l = fmaf(my, my, -b);
@@ -256,17 +258,31 @@ __device__ __forceinline__ void rec_plain(float E, float mx, float my, float mz,
     const float s1 = a + b;
     float bb = s1 - a;
     const float r1 = (a - (s1 - bb)) + (b - bb);
-    M2 = s1 + c;
+    const float M2 = s1 + c;
     bb = M2 - s1;
     const float r2 = (s1 - (M2 - bb)) + (c - bb);
-    M2lo = ((a_l + b_l) + c_l) + (r1 + r2);
+    lo = ((a_l + b_l) + c_l) + (r1 + r2);
+    return M2;
   } else {
-    M2 = fmaf(mx, mx, fmaf(my, my, mz * mz));
+    return fmaf(mx, mx, fmaf(my, my, mz * mz));
   }
+}
+// The velocity w along the sweep and the pressure p; true if clamped or vacuum.
+template <int EOS, int REC, bool CLAMP>
+__device__ __forceinline__ bool root(float E, float M2, float M2lo, float m, float omd, float B, float ec, float& w,
+                                     float& p) {
   const float E2 = E * E;
-  const float lim = omd * E;
-  ok = ok & (M2 <= lim * lim) & (E > 0.0f);
-  const float D = fmaxf(REC == fast::REC_DF ? fmaf(E, E, -M2) - M2lo : E2 - M2, 0.0f);
+  float D = REC == fast::REC_DF ? fmaf(E, E, -M2) - M2lo : E2 - M2;
+  bool cl = false;
+  if (CLAMP) {
+    const float lim = omd * E;
+    const float L2 = lim * lim;
+    cl = M2 > L2;
+    m = cl ? m * (lim * rsqrtf(M2)) : m;
+    D = cl ? E2 - L2 : D;
+    M2 = cl ? L2 : M2;
+  }
+  D = fmaxf(D, 0.0f);
   float pp;
   if constexpr (EOS == EOS_BAG) {
     const float R0 = fmaf(3.0f, D, E2);
@@ -284,6 +300,13 @@ __device__ __forceinline__ void rec_plain(float E, float mx, float my, float mz,
   }
   w = m * __fdividef(1.0f, E + pp);
   p = pp;
+  if (CLAMP) {
+    const bool vac = !(E > 0.0f);
+    w = vac ? 0.0f : w;
+    p = vac ? 0.0f : p;
+    cl = cl || vac;
+  }
+  return cl;
 }
 
 template <int EOS, int AXIS, int REC, int C, int XL, int MINB>
@@ -475,18 +498,27 @@ __global__ void __launch_bounds__(Lay<AXIS, C, XL>::WARPS * 32, MINB)
           if (cl && h == 0) nclamp += valid && (unsigned)(pos0 + c - s0) < (unsigned)(s1 - s0) ? 1u : 0u;
         }
       } else {
+        float M2[C], Ml[C];
         bool okl = true, okm = true, okr = true;
 #pragma unroll
-        for (int c = 0; c < C; ++c)
-          rec_plain<EOS, REC>(H[0][c], H[1][c], H[2][c], H[3][c], H[1 + AXIS][c], P.f_omd, P.f_bag_B, P.f_bag_ec,
-                              w[c + 1], p[c + 1], c < NG ? okl : (c >= C - NG ? okr : okm));
+        for (int c = 0; c < C; ++c) {
+          M2[c] = norm2<REC>(H[1][c], H[2][c], H[3][c], Ml[c]);
+          const float lim = P.f_omd * H[0][c];
+          bool& ok = c < NG ? okl : (c >= C - NG ? okr : okm);
+          ok = ok & (M2[c] <= lim * lim) & (H[0][c] > 0.0f);
+        }
         // the half-step values of the tile's outer three cells per side are not used
-        if (!okm || (!okl && (h == 0 || g > 0)) || (!okr && (h == 0 || g < G - 1))) {
+        const bool rare = !okm || (!okl && (h == 0 || g > 0)) || (!okr && (h == 0 || g < G - 1));
+        if (!__any_sync(0xffffffffu, rare)) {
+#pragma unroll
+          for (int c = 0; c < C; ++c)
+            root<EOS, REC, false>(H[0][c], M2[c], Ml[c], H[1 + AXIS][c], P.f_omd, P.f_bag_B, P.f_bag_ec, w[c + 1],
+                                  p[c + 1]);
+        } else {
 #pragma unroll
           for (int c = 0; c < C; ++c) {
-            const unsigned cl = fast::rec32<EOS, REC>(H[0][c], H[1][c], H[2][c], H[3][c], H[1 + AXIS][c],
-                                                      P.f_omd, P.omd, P.f_bag_B, P.f_bag_ec, P.tab, w[c + 1],
-                                                      p[c + 1]);
+            const bool cl = root<EOS, REC, true>(H[0][c], M2[c], Ml[c], H[1 + AXIS][c], P.f_omd, P.f_bag_B,
+                                                 P.f_bag_ec, w[c + 1], p[c + 1]);
             if (cl && h == 0) nclamp += valid && (unsigned)(pos0 + c - s0) < (unsigned)(s1 - s0) ? 1u : 0u;
           }
         }

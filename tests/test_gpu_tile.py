@@ -95,3 +95,28 @@ def test_small_batches_by_event_match_streaming_bitwise(monkeypatch, precision, 
         assert sa == sb and ca == cb > 0
         for x, y in zip(ua, ub):
             assert np.array_equal(x, y)
+
+
+@pytest.mark.parametrize("precision,eos", [("fp32", "ideal"), ("fp32", "bag"), ("fp32", "table"), ("mixed", "ideal"),
+                                           ("mixed", "bag"), ("mixed_fp64", "ideal")])
+@pytest.mark.parametrize("share", [0.002, 0.4])
+def test_many_clamped_and_vacuum_cells_bitwise(monkeypatch, precision, eos, share):
+    """Warps with a few and with many cells of |M| > E, E = 0 and E < 0, in the
+    tiles' own cells, halos and outermost cells: states and counts as streamed,
+    also with the atomics of a warp's lanes added up."""
+    require_gpu()
+    kw = dict(precision=precision, eos=eos)
+    if eos == "table":
+        kw.update(table=TABLE, table_de=0.01)
+    for i, shape in enumerate([(131, 33, 20), (30, 101, 120), (200, 7, 69)]):
+        pr = W.random_state(shape, seed=i, vmax=0.6, e_range=(0.3, 3.0))
+        U = oracle().prim2cons(OR.params(shape), *pr.as_list())
+        pick = np.random.default_rng(i).random(U[0].shape)
+        U[2][pick < share] = -2.0 * U[0][pick < share]
+        U[0][pick > 1 - share / 4] *= 0.0
+        U[0][pick > 1 - share / 8] = -0.1
+        ref = run(monkeypatch, "off", shape, U, **kw)
+        got = run(monkeypatch, "", shape, U, **kw)
+        assert got[1] == ref[1] > share * U[0].size, shape
+        for a, b in zip(ref[0], got[0]):
+            assert np.array_equal(a, b, equal_nan=True), shape
