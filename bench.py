@@ -114,7 +114,7 @@ def measured_peak():
 def kernel_source_hash():
     h = hashlib.sha256()
     for f in ("sweep.cuh", "sweep_fast.cuh", "sweep_launch.cuh", "sweep_f32.cu",
-              "sweep_mixed.cu", "sweep_f64.cu"):
+              "sweep_mixed.cu", "sweep_f64.cu", "sweep_tile.cuh", "tile_plan.h"):
         with open(os.path.join(ROOT, "paper_1206_0919_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]

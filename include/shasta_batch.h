@@ -4,11 +4,14 @@
  * A batch keeps the state of many events in one device pool and advances
  * every resident event with one launch per sweep axis over a work list of
  * its events (work units: whole line groups, or equal ranges of positions
- * that may cut lines), instead of one launch per event and sweep.  The paper weighs the size of a kernel's working set against the
- * cost of orchestrating many kernel calls from the host (Sec. 3.1.2) and
- * enqueues the sweeps of one grid from a host loop (Sec. 3.1.3); here the
- * work of all events of a sweep shares a launch, and six steps of launches
- * are replayed as one CUDA graph while the batch does not change.
+ * that may cut lines), instead of one launch per event and sweep.  The paper
+ * weighs the size of a kernel's working set against the cost of orchestrating
+ * many kernel calls from the host (Sec. 3.1.2) and enqueues the sweeps of one
+ * grid from a host loop (Sec. 3.1.3); here the work of all events of a sweep
+ * shares a launch (up to eight events too small to fill the streaming sweep
+ * take the tiled sweep of single contexts, a launch each, instead), and six
+ * steps of launches are replayed as one CUDA graph while the batch does not
+ * change.
  *
  * Every event is advanced exactly as a single context with the same grid,
  * boundary rule, EoS, lambda and options would advance it (shasta.h): the
