@@ -520,11 +520,11 @@ void drop_graph(shasta_ctx* c) {
 
 // Time of one sweep of axis with parameters P, on tiles or streamed, from the
 // current buffer into the other one: one launch after an untimed one (two
-// runs of a choice differ by 0.1% at 0.1 ms and more), five of short ones.
+// runs of a choice differ by 0.1% at 0.1 ms and more), three of short ones.
 cudaError_t time_choice(shasta_ctx* c, int axis, bool tile, SweepParams P, cudaEvent_t e0, cudaEvent_t e1, float& ms) {
   P.clamp_count = nullptr;  // trial sweeps are no steps: their clamps do not count
   cudaError_t ce = tile ? launch_tile(c, axis, P) : launch_params(c, axis, P);
-  for (int reps = 1; reps <= 5 && ce == cudaSuccess; reps += 4) {
+  for (int reps = 1; reps <= 3 && ce == cudaSuccess; reps += 2) {
     ce = cudaEventRecord(e0, c->stream);
     for (int r = 0; r < reps && ce == cudaSuccess; ++r)
       ce = tile ? launch_tile(c, axis, P) : launch_params(c, axis, P);

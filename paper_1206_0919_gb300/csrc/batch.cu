@@ -586,17 +586,20 @@ shasta_status autotune(shasta_batch* b) {
     float best = 1e30f;
     int bv = 0;
     double bsh = b->tune_share[a];
-    // one sweep of every event per choice after an untimed one, three where
-    // that is short (the first choice tells; two runs of a choice differ by
-    // 0.1% at 0.1 ms and more); the other register variant for the best share
-    // only.  Every trial is time taken from the batch's own steps: 32 sweeps an
-    // axis were a third of a 48-step batch, these are 10, or 21 short ones.
+    // one sweep of every event per choice, three where that is short (the
+    // first choice tells; two runs of a choice differ by 0.1% at 0.1 ms and
+    // more); the other register variant for the best share only.  An untimed
+    // one goes before where it matters: short sweeps, and a kernel that may not
+    // be loaded yet.  Every trial is time taken from the batch's own steps: 32
+    // sweeps an axis were a third of a 48-step batch, these are 7, or 21 short
+    // ones.
     int reps = 1;
     auto trial = [&](int var, double sh) {
       const int vars[3] = {var, var, var};
       const double shs[3] = {sh, sh, sh};
       fit_ranges(b, recs, vars, shs);
-      cudaError_t ce = launch_slot(b, recs, b->cur);
+      cudaError_t ce = cudaSuccess;
+      if (reps > 1 || var != 0 || best == 1e30f) ce = launch_slot(b, recs, b->cur);
       float ms = 0;
       while (ce == cudaSuccess) {
         ce = cudaEventRecord(e0, b->stream);
