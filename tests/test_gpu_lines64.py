@@ -69,3 +69,24 @@ def test_lines_match_streaming_bitwise(monkeypatch, eos, bc):
                 assert got[1] == ref[1] > 0, (shape, wild, lines)
                 for a, b in zip(ref[0], got[0]):
                     assert np.array_equal(a, b, equal_nan=True), (shape, wild, lines)
+
+
+@pytest.mark.parametrize("de", [0.01, 2.0 ** -40, 0.3])
+def test_table_index_and_fraction_at_the_nodes(monkeypatch, de):
+    """The index and fraction taken from the bit pattern give what the
+    conversions give: energies on, one ulp below and above a table's nodes,
+    below the first interval's end, above the table and far above it."""
+    require_gpu()
+    table = np.arange(40) * de * 0.25
+    k = np.arange(1, 60) * de
+    e = np.concatenate([k, np.nextafter(k, 0), np.nextafter(k, 1e9), de * 10.0 ** -np.arange(1, 20), de * 2.0 ** np.arange(5, 40)])
+    shape = (e.size, 4, 3)
+    U = [np.broadcast_to(e, (3, 4, e.size)).copy() for _ in range(5)]
+    for j, f in enumerate((0.0, 0.3, -0.2)):
+        U[1 + j] = f * U[0] * (np.arange(4) % 2)[None, :, None]
+    kw = dict(eos="table", table=table, table_de=de)
+    ref = run(monkeypatch, "off", shape, U, 3, **kw)
+    got = run(monkeypatch, None, shape, U, 3, **kw)
+    assert got[1] == ref[1]
+    for a, b in zip(ref[0], got[0]):
+        assert np.array_equal(a, b, equal_nan=True)
