@@ -341,8 +341,12 @@ static __device__ __noinline__ bool rec64_over(double E, double M2, double omd) 
 // The same bits for a physical, unclamped cell with a normal E: bound by the
 // double pipe (2 operations per SM and clock), so the quotients and the root
 // are the short ones, comparisons and conversions integer operations, and the
-// clamp is compared exactly only within 1/32 of E^2: 28 double operations for
-// the ideal gas instead of about 65.
+// clamp is compared exactly only where M^2 is near E^2: 28 double operations
+// for the ideal gas instead of about 65.  Near means a high word above that of
+// E^2 less 0x10000, which is 1/32 of E^2 at least (a high word is 2^-20 of a
+// significand of 1 and 2^-21 of one near 2, and the step into the binade below
+// halves it once more; 0x8000 would leave 1/64), and a margin delta of up to
+// 0.01 needs 1 - 0.99^2 = 0.0199; larger ones are always compared exactly.
 template <int EOS>
 __device__ __forceinline__ unsigned rec64(float Ef, float mxf, float myf, float mzf, float m1f,
                                           double omd, double B, double ec, float& w, float& p) {
@@ -350,7 +354,7 @@ __device__ __forceinline__ unsigned rec64(float Ef, float mxf, float myf, float 
     const double E = f64::widen(Ef), mx = f64::widen(mxf), my = f64::widen(myf), mz = f64::widen(mzf);
     const double M2 = fma(mx, mx, fma(my, my, mz * mz));
     const double E2 = E * E;
-    if (!((f64::hi(M2) > f64::hi(E2) - 0x8000 || f64::hi(omd) < 0x3fefae15) && rec64_over(E, M2, omd))) {
+    if (!((f64::hi(M2) > f64::hi(E2) - 0x10000 || f64::hi(omd) < 0x3fefae15) && rec64_over(E, M2, omd))) {
       double D = fma(E, E, -M2);
       if (f64::hi(D) < 0) D = 0.0;
       double pp;
