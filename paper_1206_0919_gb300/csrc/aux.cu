@@ -242,13 +242,16 @@ __device__ __forceinline__ bool finite(double x) { return f64::mag(x) < 0x7ff000
 __device__ __forceinline__ bool negative(double x) { return f64::hi(x) < 0 && !f64::is_zero(x); }
 
 // Whether x^2 + y^2 + z^2 is below (1 - 2^-16) a^2, decided in FP32 on the
-// significands cut to 24 bits and scaled by a's exponent (a > 0, normal): a
-// true answer is certain, a false one leaves the question to the double form.
+// significands cut to 24 bits and scaled by a's exponent: a true answer is
+// certain, a false one leaves the question to the double form.  That form
+// compares rounded squares, which answers otherwise where both overflow or
+// fall among the subnormals (there 2^-16 is no longer above their rounding,
+// from a = 2^-528 down), so such an a is left to it as well.
 __device__ __forceinline__ bool clearly_below(double x, double y, double z, double a) {
   const unsigned ha = f64::mag(a), ea = ha >> 20;
   const float fa = __uint_as_float(0x3f800000u | ((ha & 0xfffffu) << 3) | ((unsigned)__double2loint(a) >> 29));
   float s = 0.0f;
-  bool big = f64::hi(a) < (1 << 20);
+  bool big = f64::hi(a) < 0 || !f64::within<-500, 511>(a);
   const double c[3] = {x, y, z};
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
