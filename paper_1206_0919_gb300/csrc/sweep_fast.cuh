@@ -332,13 +332,20 @@ __device__ __noinline__ unsigned rec64_rest(float Ef, float mxf, float myf, floa
   return clamped;
 }
 
-// Whether |M| exceeds (1 - delta) E (out of line: asked near |v| = 1 only).
-static __device__ __noinline__ bool rec64_over(double E, double M2, double omd) {
+// The clamp of rec64, out of line (asked near |v| = 1 only; inlined, the
+// compiler predicates it and every cell pays): the momentum along the sweep and
+// |M|^2 as they are where |M| <= (1 - delta) E, else m scaled to the limit and
+// its square; an infinite or NaN |M|^2 comes back as NaN.
+static __device__ __noinline__ double2 rec64_clamp(double E, double M2, double m, double omd) {
   const double lim = omd * E;
-  return !(M2 <= lim * lim);
+  const double L2 = lim * lim;
+  if (M2 <= L2) return make_double2(m, M2);
+  if (f64::mag(M2) >= 0x7ff00000u) return make_double2(m, __hiloint2double(0x7ff80000, 0));
+  const double M = f64::sqrt_raw(M2);
+  return make_double2(m * f64::quot_raw(lim, M, f64::recip_raw(M)), L2);
 }
 
-// The same bits for a physical, unclamped cell with a normal E: bound by the
+// The same bits for a cell with a normal E and finite momenta: bound by the
 // double pipe (2 operations per SM and clock), so the quotients and the root
 // are the short ones, comparisons and conversions integer operations, and the
 // clamp is compared exactly only where M^2 is near E^2: 28 double operations
@@ -347,14 +354,30 @@ static __device__ __noinline__ bool rec64_over(double E, double M2, double omd) 
 // significand of 1 and 2^-21 of one near 2, and the step into the binade below
 // halves it once more; 0x8000 would leave 1/64), and a margin delta of up to
 // 0.01 needs 1 - 0.99^2 = 0.0199; larger ones are always compared exactly.
+// Clamped cells and vacuum stay on the short forms: evolved hot spots hold 3%
+// of them, and where they went through rec64_rest most warps ran both (step
+// 120, us a step: 128^3 1713, 1031 so; 160^3 3566, 2065; 200^3 5832, 3616).
 template <int EOS>
 __device__ __forceinline__ unsigned rec64(float Ef, float mxf, float myf, float mzf, float m1f,
                                           double omd, double B, double ec, float& w, float& p) {
+  if ((int)__float_as_uint(Ef) <= 0) {  // E <= 0
+    w = 0.0f;
+    p = 0.0f;
+    return 1;
+  }
   if (__float_as_uint(Ef) - 0x00800000u < 0x7f000000u) {
     const double E = f64::widen(Ef), mx = f64::widen(mxf), my = f64::widen(myf), mz = f64::widen(mzf);
-    const double M2 = fma(mx, mx, fma(my, my, mz * mz));
+    double M2 = fma(mx, mx, fma(my, my, mz * mz));
+    double m = f64::widen(m1f);
     const double E2 = E * E;
-    if (!((f64::hi(M2) > f64::hi(E2) - 0x10000 || f64::hi(omd) < 0x3fefae15) && rec64_over(E, M2, omd))) {
+    unsigned clamped = 0;
+    if (f64::hi(M2) > f64::hi(E2) - 0x10000 || f64::hi(omd) < 0x3fefae15) {
+      const double2 t = rec64_clamp(E, M2, m, omd);
+      clamped = f64::bits(t.y) != f64::bits(M2) ? 1u : 0u;
+      m = t.x;
+      M2 = t.y;
+    }
+    if (f64::mag(M2) < 0x7ff00000u) {
       double D = fma(E, E, -M2);
       if (f64::hi(D) < 0) D = 0.0;
       double pp;
@@ -373,10 +396,9 @@ __device__ __forceinline__ unsigned rec64(float Ef, float mxf, float myf, float 
         pp = f64::quot_raw(D, se, f64::recip_raw(se));
       }
       const double h = E + pp;
-      const double m = f64::widen(m1f);
       w = m1f == 0.0f ? m1f : f64::narrow<float>(f64::quot_raw(m, h, f64::recip_raw(h)));
       p = f64::narrow<float>(pp);
-      return 0;
+      return clamped;
     }
   }
   return rec64_rest<EOS>(Ef, mxf, myf, mzf, m1f, omd, B, ec, w, p);

@@ -59,3 +59,40 @@ def test_clamp_margin_against_double(monkeypatch, delta, eos, tile):
         ref = oracle().sweep(P, U, axis)
         for g, r in zip(got, ref):
             assert np.max(np.abs(g - r) / U[0]) <= 1e-5, axis
+
+
+@pytest.mark.parametrize("tile", ["", "off"])
+@pytest.mark.parametrize("eos", [OR.EOS_IDEAL, OR.EOS_BAG])
+@pytest.mark.parametrize("scale", [1.0, 1e-30, 1e18])
+def test_clamped_cells_against_oracle(monkeypatch, scale, eos, tile):
+    """States of which most cells are clamped, |M| up to 3 E, at energies whose
+    squares leave the range of float, against the oracle (the bound above, with
+    |M| in the place of E); cells of E = 0 and E < 0 among them are counted."""
+    require_gpu()
+    monkeypatch.setenv("SHASTA_TILE", tile)
+    nx, ny, nz = SHAPE
+    U, _ = state(0.01, eos)
+    x = np.arange(nx)[None, None, :] / nx
+    U = [U[0] * scale] + [(m * scale * (1.7 + 1.3 * np.sin(4 * np.pi * x))) for m in U[1:4]] + [U[0].copy()]
+    U = [u.astype(np.float32).astype(np.float64) for u in U]
+    over = int((U[1] ** 2 + U[2] ** 2 + U[3] ** 2 > ((1 - 1e-6) * U[0]) ** 2).sum())
+    assert over > U[0].size // 3
+    P = OR.params(SHAPE, bc=OR.BC_PERIODIC, eos=eos, delta=1e-6)
+    kw = dict(precision="mixed_fp64", bc="periodic", eos="bag" if eos else "ideal", check_input=False, autotune=False)
+    with S.Solver(SHAPE, **kw) as s:
+        for axis in range(3):
+            s.set_conserved(U)
+            s.sweep(axis)
+            got = s.get_conserved()
+            assert s.counters() == over, axis
+            ref = oracle().sweep(P, U, axis)
+            for k, (g, r) in enumerate(zip(got, ref)):
+                assert np.max(np.abs(g - r) / (3 * U[0] / (scale if k == 4 else 1.0))) <= 1e-5, axis
+        V = [u.copy() for u in U]
+        V[0][:, ::7, 3::11] = 0.0
+        V[0][:, 1::9, 5::13] *= -1.0
+        M2 = V[1] ** 2 + V[2] ** 2 + V[3] ** 2
+        bad = (V[0] <= 0) | (M2 > ((1 - 1e-6) * V[0]) ** 2)
+        s.set_conserved(V)
+        s.sweep(0)
+        assert s.counters() == int(bad.sum())
