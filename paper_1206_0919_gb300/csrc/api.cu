@@ -388,7 +388,22 @@ long long stream_share(const shasta_ctx* c, int axis) {
 // results through shared memory as well, tiles stay ahead (200^3, 137: 116
 // against 90; 256^3, 288: 211 against 197).  In between the autotuner times
 // both.
+// Short lines and MIXED_FP64 need the estimates of tile_plan.h in favour of
+// tiles as well: untuned the lesser time, tuned tiles untimed only where they
+// take less than kTileSure of the streamed time.  (A step on 512 x 512 x 4
+// cells, us: tiles 247, streamed 127; on 512 x 512 x 1 228 and 103.)
 constexpr long long kTileAlways = 40, kTileShare = 64;
+constexpr double kTileSure = 0.7;
+
+bool tile_rule(const shasta_ctx* c, int axis, bool sure) {
+  const int n = axis == 0 ? c->g.nx : (axis == 1 ? c->g.ny : c->g.nz);
+  const bool rec64 = c->o.precision == SHASTA_MIXED_FP64;
+  const long long share = stream_share(c, axis);
+  if (sure ? share >= kTileAlways : axis != 0 && share >= kTileShare) return false;
+  if (!by_cost(n, rec64)) return true;
+  const SweepCost k = sweep_cost((long long)c->ncell / n, n, axis, c->tile[axis].shape, rec64, c->sm_count);
+  return sure ? k.tile <= kTileSure * k.stream : k.tile <= k.untimed;
+}
 
 // Launch choice for an axis: environment overrides, else the autotuned
 // choice, else (FP32 / MIXED) tiles or variant 0 with one range per resident
@@ -402,7 +417,7 @@ Choice launch_choice(const shasta_ctx* c, int axis) {
     return h;
   }
   if (c->tile[axis].shape >= 0) {
-    h.tile = c->force_tile >= 0 || (c->tuned ? c->tune_tile[axis] : axis == 0 || stream_share(c, axis) < kTileShare);
+    h.tile = c->force_tile >= 0 || (c->tuned ? c->tune_tile[axis] : tile_rule(c, axis, false));
     if (h.tile) return h;
   }
   h.variant = c->tuned ? c->tune_var[axis] : 0;
@@ -539,8 +554,8 @@ cudaError_t time_choice(shasta_ctx* c, int axis, bool tile, SweepParams P, cudaE
 
 // Times candidate launch choices per axis with repeated sweeps from the
 // current buffer into the other one (the state itself is not changed) and
-// keeps the fastest.  FP32 / MIXED: tiles (alone, untimed, where a warp's
-// streamed share is under kTileAlways), or ranges of one line group (no line is
+// keeps the fastest.  FP32 / MIXED: tiles (alone, untimed, where tile_rule
+// is sure of them), or ranges of one line group (no line is
 // cut) or of 1/2 .. 2 ranges per resident warp, and the best of them with the
 // other register variant.
 // FP64: nothing to time on whole lines in shared memory; else the line segment
@@ -568,7 +583,7 @@ shasta_status autotune(shasta_ctx* c) {
     double bsh = 0.0;
     if (f64 && c->lines[axis].B > 0) continue;
     if (c->tile[axis].shape >= 0) {
-      if (c->force_tile >= 0 || stream_share(c, axis) < kTileAlways) {
+      if (c->force_tile >= 0 || tile_rule(c, axis, true)) {
         c->tune_tile[axis] = true;
         continue;
       }

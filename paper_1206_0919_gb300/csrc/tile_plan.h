@@ -1,5 +1,8 @@
-// tile_plan.h -- which tile shape a line takes (host code, no CUDA).
+// tile_plan.h -- which tile shape a line takes, and where tiles are worth it
+// (host code, no CUDA).
 #pragma once
+
+#include <algorithm>
 
 namespace shasta {
 
@@ -51,5 +54,49 @@ inline int tile_shape_for(int n, int axis) {
   }
   return best;
 }
+
+// Estimated times (us, 152 SMs) of one sweep over `lines` lines of n cells: on
+// tiles, streamed with a timed choice of ranges, and streamed untimed (ranges
+// of at least 24 positions, so lines shorter than that are taken one after the
+// other by a warp).  A tile computes all its positions, own or not, so short
+// lines waste most of it (a line of 16 cells: 64 positions), where streaming
+// pays a lead-in of 14 to 26 positions; the double recovery (rec64) makes each
+// position ten times dearer in both.  g: line groups per warp of one wave of 16
+// per SM; below one the streamed chain is bound by its latency.
+// Measured against (x, FP32, us, tiles / timed / untimed): 200 x 200 lines of 8
+// cells 33.7 / 25.5 / 47.9, of 24 33.5 / 37.7 / 37.8; 400 x 400 of 5 143 / 66 /
+// 89, of 16 116 / 87 / 87, of 32 114 / 121 / 120; 1024 x 1024 of 1 908 / 295 /
+// 390, of 16 780 / 509 / 511, of 48 771 / 871 / 877; z is 12% faster streamed.
+// MIXED_FP64: 128 x 96 of 16 94 / 99 / 172; 200 x 200 of 16 291 / 182 / 220, of
+// 128 627 / 677 / 699; 256 x 256 of 256 2023 / 1906 / 1919; 1024 x 1024 of 16
+// 7588 / 3044 / 3141.
+struct SweepCost {
+  double tile, stream, untimed;
+};
+inline SweepCost sweep_cost(long long lines, int n, int axis, int shape, bool rec64, int sm_count) {
+  const double g = (double)lines / (512.0 * sm_count);
+  const long long cut = ((long long)n + tile_own(shape) - 1) / tile_own(shape);
+  const double computed = (double)(cut * tile_positions(shape));
+  const double below = std::min(g, 1.0);
+  const double queue = n < 24 ? (double)((23 + n) / n) : 1.0;  // lines one after the other
+  SweepCost c;
+  if (rec64) {
+    const double per = 8.5 * g + (2.2 - 1.5 * below) * std::min(1.0, 48.0 / n);
+    c.tile = 10.0 + 8.5 * g * computed;
+    c.stream = (n + 14) * per;
+    c.untimed = (n + 14) * std::max(per, queue > 1.0 ? 3.3 * queue : 0.0);
+  } else {
+    const double dir = axis == 0 ? 1.0 : 0.88;
+    const double per = dir * std::max(0.6 + 0.6 * below * below, g);
+    // lines shorter than the halo take the tile's general ghost mapping
+    c.tile = 4.0 + 0.85 * g * computed * (n < 6 ? 1.2 : 1.0);
+    c.stream = (n + 26) * per;
+    c.untimed = (n + 26) * std::max(per, queue > 1.0 ? 0.48 * dir * queue : 0.0);
+  }
+  return c;
+}
+// Where the choice between tiles and streaming goes by these estimates too:
+// lines that leave most of a tile unused, and the double recovery at any size.
+inline bool by_cost(int n, bool rec64) { return rec64 || n < 50; }
 
 }  // namespace shasta
