@@ -354,7 +354,11 @@ void fit_ranges(const shasta_batch* b, std::vector<LaunchRec>& V, const int var[
 // Few events of few positions take the tiled kernels, each event in launches
 // of its own: below about 40 positions per resident warp the streaming sweep is
 // bound by its serial chain (one 64^3 event: 27 us a sweep, tiled 8.4), and up
-// to eight events the launches cost less than that.
+// to eight events the launches cost less than that (16^3, us a step, step by
+// step: one event 60 streamed, 11 tiled; eight 62 and 52).  With lines that
+// leave most of a tile unused the positions computed decide: the sum of the
+// tiled times against the streamed chain and its throughput (1 x 512 x 512, us a
+// step: 125 streamed, 247 tiled).
 constexpr long long kTilePositions = 40;
 constexpr int kTileEvents = 8;
 
@@ -362,7 +366,26 @@ bool wants_tiles(const shasta_batch* b) {
   if (b->tiles_off || b->force_range >= 0 || b->nlive > kTileEvents) return false;
   for (int a = 0; a < 3; ++a)
     if (total_positions(b, a) >= kTilePositions * warp_slots(b, 0, a, 0)) return false;
-  return true;
+  bool some_short = false;
+  double tiled = 0.0, streamed = 0.0;
+  for (int a = 0; a < 3; ++a) {
+    double chain = 0.0, flow = 0.0, floor = 0.0, work = 0.0;
+    for (const Event& e : b->ev) {
+      if (!e.live) continue;
+      const int n = extent(e.g, a);
+      const long long lines = plane_of(e.g, a);
+      some_short = some_short || by_cost(n, false);
+      const int shape = tile_shape_for(n, a);
+      floor = sweep_cost(0, n, a, shape, false, b->sm_count).tile;
+      work += sweep_cost(lines, n, a, shape, false, b->sm_count).tile - floor;  // (side by side)
+      // (long lines are cut into ranges)
+      chain = std::max(chain, sweep_cost(lines, std::min(n, 40), a, 0, false, b->sm_count).stream);
+      flow += (double)(n + 26) * (double)lines / (512.0 * b->sm_count);
+    }
+    tiled += floor + work;
+    streamed += std::max(chain, flow);
+  }
+  return !some_short || tiled <= streamed;
 }
 
 TilePlan tile_of(const shasta_batch* b, const Event& e, int axis) {
