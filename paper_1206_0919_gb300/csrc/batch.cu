@@ -47,6 +47,7 @@ struct LaunchRec {
   size_t idx_off = 0, pre_off = 0, gpre_off = 0;  // event indices, position / group prefixes
   long long items = 0;   // (line group, position) pairs
   long long groups = 0;  // line groups
+  int longest = 0;       // cells of the longest line
   int variant = 0;       // register variant and positions per work range
   long long range = 0;   // (0: whole line groups)
 };
@@ -310,6 +311,7 @@ LaunchRec make_list(const shasta_batch* b, std::vector<int> ids, int axis, int e
   L.axis = axis;
   L.eos = eos;
   L.nlist = (int)ids.size();
+  L.longest = extent(b->ev[ids[0]].g, axis);
   L.idx_off = out.size();
   for (int i : ids) out.push_back(i);
   L.pre_off = out.size();
@@ -333,21 +335,39 @@ LaunchRec make_list(const shasta_batch* b, std::vector<int> ids, int axis, int e
 
 // Sets the variants and range lengths of the launches of one sweep slot: for
 // a launch by itself `share` ranges per resident warp; several launches (both
-// EoS, or events at different phases) always take whole line groups.  Ranges
+// EoS, or events at different phases) take whole line groups.  Ranges
 // fill an SM with one long round of warps, and beside a second kernel that
 // round slows to less than half (192^3 ideal, 128^3 bag, 64^3 of each: 826 us a
 // step with ranges cut for both together, 559 with ranges for each, 397 with
 // line groups; 64^3 three of each 338 against 169; 160^3 of each 454 against
-// 374), while many short units let one kernel follow the other.
+// 374; three 128^3 at different phases 786 against 305), while many short units
+// let one kernel follow the other.  Lines that outlast the others' work are no
+// such units: where the longest passes 2.5 times the slot's positions per
+// resident warp, or 6 times in small slots, lines are cut into ranges of half
+// of that share.  Us a step, line groups -> ranges: twelve 16 x 16 x 1024 of
+// both EoS 638 -> 308, at different phases 1067 -> 287; 64 x 64 x 2000 of each
+// 1361 -> 800; 100 x 100 x 800 of each 945 -> 752; 192^3 and 16 x 16 x 1500 824
+// -> 336; small slots, twelve 100 x 20 x 20 at different phases (11.7 shares)
+// 155 -> 121, nine 30 x 30 x 120 (7) 161 -> 120.  Below the line: twelve 48^3 at
+// different phases (2.1 shares) 127 against 268 cut, six 200 x 200 x 20 (2.4)
+// 332 against 465, ten 40^3 of both EoS (3.6) 112 against 187.
+bool long_lines(double longest, double each) {
+  return longest > std::max(2.5 * each, std::max(std::min(6.0 * each, 160.0), 30.0));
+}
+
 void fit_ranges(const shasta_batch* b, std::vector<LaunchRec>& V, const int var[3], const double share[3]) {
+  long long items = 0;
+  for (const LaunchRec& L : V) items += L.items;
   for (LaunchRec& L : V) {
     L.variant = var[L.axis];
+    const long long warps = warp_slots(b, L.eos, L.axis, L.variant);
+    const double each = (double)items / (double)warps;
     if (b->force_range >= 0)
       L.range = b->force_range;
+    else if (V.size() == 1)
+      L.range = share[L.axis] > 0.0 ? range_for(L.items, warps, share[L.axis]) : 0;
     else
-      L.range = share[L.axis] > 0.0 && V.size() == 1
-                    ? range_for(L.items, warp_slots(b, L.eos, L.axis, L.variant), share[L.axis])
-                    : 0;
+      L.range = long_lines(L.longest, each) ? std::max(24LL, (long long)(0.5 * each) + 1) : 0;
   }
 }
 

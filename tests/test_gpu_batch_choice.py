@@ -1,6 +1,8 @@
 """Which launches a batch takes (launches per step) and that the choice changes
 no bit: few small events tiled launches of their own, events whose lines would
 leave most of a tile unused the shared streaming launches."""
+import time
+
 import numpy as np
 import pytest
 
@@ -42,3 +44,38 @@ def test_thin_events_stream(monkeypatch, shape, tiles):
     got = batch(events, 8)
     assert got[2]["launches_per_step"] == (6 if tiles else 3)
     assert same(ref, got)
+
+
+def us_per_step(b, n=12):
+    best = 1e9
+    b.step(n)
+    b.sync()
+    for _ in range(5):
+        t = time.perf_counter()
+        b.step(n)
+        b.sync()
+        best = min(best, time.perf_counter() - t)
+    return best / n * 1e6
+
+
+@pytest.mark.parametrize("shape,count,ahead", [((16, 16, 1024), 12, 0), ((1024, 16, 16), 12, 1), ((12, 700, 20), 10, 0)])
+def test_long_lines_are_cut_beside_other_launches(monkeypatch, shape, count, ahead):
+    """Long lines of several launches in a slot (two equations of state, events
+    at different phases) are cut into ranges: the bits of whole line groups, in
+    well under the time of those (measured at 0.3 to 0.6 of it)."""
+    require_gpu()
+    events = [(shape, "ideal" if ahead or i % 2 else "bag", ahead) for i in range(count)]
+    res, us = [], []
+    for forced in ("0", None):  # whole line groups, the rule
+        if forced:
+            monkeypatch.setenv("SHASTA_BATCH_RANGE", forced)
+        else:
+            monkeypatch.delenv("SHASTA_BATCH_RANGE")
+        res.append(batch(events, 8, autotune=False))
+        with S.Batch(count * int(np.prod(shape)) + 64 * count, autotune=False) as b:
+            for i, (sh, eos, n) in enumerate(events):
+                b.add_primitives(sh, prims(sh, i), eos=eos)
+                b.step(n)
+            us.append(us_per_step(b))
+    assert same(*res)
+    assert us[1] < 0.8 * us[0], us
