@@ -52,6 +52,14 @@ struct LaunchRec {
   long long range = 0;   // (0: whole line groups)
 };
 
+// Launch choice per axis: register variant; ranges per resident warp of a
+// launch by itself (0: whole line groups); of the two equations of state's
+// launches together (0: line groups, -1: by the rule of fit_ranges).
+struct LaunchTune {
+  int var[3] = {0, 0, 0};
+  double share[3] = {0, 0, 0}, pair[3] = {-1, -1, -1};
+};
+
 }  // namespace
 
 struct shasta_batch {
@@ -93,8 +101,7 @@ struct shasta_batch {
   // launch choice per axis: register variant and ranges per resident warp
   bool tuned = false;
   long long force_range = -1;  // >= 0: work range of every axis (environment override; 0 = line groups)
-  int tune_var[3] = {0, 0, 0};
-  double tune_share[3] = {0, 0, 0};  // ranges per resident warp; 0: whole line groups
+  LaunchTune tune;
   // few small events: every event sweeps by the tiled kernels in launches of
   // its own (resident blocks per SM of the kernels readied so far)
   bool by_event = false;
@@ -195,8 +202,9 @@ long long total_groups(const shasta_batch* b, int axis) {
 void model_choice(shasta_batch* b) {
   for (int a = 0; a < 3; ++a) {
     const long long warps = warp_slots(b, 0, a, 0);
-    b->tune_var[a] = 0;
-    b->tune_share[a] = total_groups(b, a) >= 2 * warps ? 0.0 : 1.0;
+    b->tune.var[a] = 0;
+    b->tune.share[a] = total_groups(b, a) >= 2 * warps ? 0.0 : 1.0;
+    b->tune.pair[a] = -1.0;
   }
 }
 
@@ -355,17 +363,19 @@ bool long_lines(double longest, double each) {
   return longest > std::max(2.5 * each, std::max(std::min(6.0 * each, 160.0), 30.0));
 }
 
-void fit_ranges(const shasta_batch* b, std::vector<LaunchRec>& V, const int var[3], const double share[3]) {
+void fit_ranges(const shasta_batch* b, std::vector<LaunchRec>& V, const LaunchTune& t) {
   long long items = 0;
   for (const LaunchRec& L : V) items += L.items;
   for (LaunchRec& L : V) {
-    L.variant = var[L.axis];
+    L.variant = t.var[L.axis];
     const long long warps = warp_slots(b, L.eos, L.axis, L.variant);
     const double each = (double)items / (double)warps;
     if (b->force_range >= 0)
       L.range = b->force_range;
     else if (V.size() == 1)
-      L.range = share[L.axis] > 0.0 ? range_for(L.items, warps, share[L.axis]) : 0;
+      L.range = t.share[L.axis] > 0.0 ? range_for(L.items, warps, t.share[L.axis]) : 0;
+    else if (V.size() == 2 && V[0].axis == V[1].axis && t.pair[L.axis] >= 0.0)
+      L.range = t.pair[L.axis] > 0.0 ? range_for(items, warps, t.pair[L.axis]) : 0;
     else
       L.range = long_lines(L.longest, each) ? std::max(24LL, (long long)(0.5 * each) + 1) : 0;
   }
@@ -461,7 +471,7 @@ shasta_status build_plan(shasta_batch* b) {
         for (int k = 0; k < 2; ++k)
           if (!groups[a][k].empty())
             b->plan[r][s].push_back(make_list(b, groups[a][k], a, k, host));
-      fit_ranges(b, b->plan[r][s], b->tune_var, b->tune_share);
+      fit_ranges(b, b->plan[r][s], b->tune);
     }
   b->by_event = wants_tiles(b);
   if (b->by_event) CK(prepare_tiles(b), "prepare tiled kernels");
@@ -606,13 +616,22 @@ cudaError_t launch_step(shasta_batch* b, int r, int ahead, bool single) {
 // changed).  The launch choice does not change results.
 shasta_status autotune(shasta_batch* b) {
   if (!b->nlive) return SHASTA_OK;
-  static const double shares[] = {0.0, 0.5, 1.0, 2.0};
+  static const double shares[] = {0.0, 0.5, 1.0, 2.0}, pairs[] = {-1.0, 0.0, 0.5, 1.0, 2.0};
   const int64_t launches0 = b->launches;  // trial launches are not counted
   cudaEvent_t e0, e1;
   CK(cudaEventCreate(&e0), "cudaEventCreate");
   CK(cudaEventCreate(&e1), "cudaEventCreate");
   shasta_status st = SHASTA_OK;
   const int n = slots_in_use(b);
+  // events at different phases share their slots with launches along other
+  // axes, which no share timed here holds for: their variant only is timed
+  bool in_step = true;
+  int64_t phase = -1;
+  for (const Event& e : b->ev)
+    if (e.live) {
+      in_step = in_step && (phase < 0 || phase == e.steps % 6);
+      phase = e.steps % 6;
+    }
   for (int a = 0; a < 3 && st == SHASTA_OK; ++a) {
     std::vector<int> host;
     std::vector<LaunchRec> recs;
@@ -627,22 +646,25 @@ shasta_status autotune(shasta_batch* b) {
     b->trial = false;
     if (st != SHASTA_OK) break;
     float best = 1e30f;
-    int bv = 0;
-    double bsh = b->tune_share[a];
+    LaunchTune pick = b->tune;
+    std::vector<std::vector<long long>> seen;  // (variant, ranges) of the choices timed so far
     // one sweep of every event per choice, three where that is short (the
     // first choice tells; two runs of a choice differ by 0.1% at 0.1 ms and
-    // more); the other register variant for the best share only.  An untimed
+    // more); choices that come to the same launches once; the other register
+    // variant for the best share only.  An untimed
     // one goes before where it matters: short sweeps, and a kernel that may not
     // be loaded yet.  Every trial is time taken from the batch's own steps: 32
     // sweeps an axis were a third of a 48-step batch, these are 7, or 21 short
     // ones.
     int reps = 1;
-    auto trial = [&](int var, double sh) {
-      const int vars[3] = {var, var, var};
-      const double shs[3] = {sh, sh, sh};
-      fit_ranges(b, recs, vars, shs);
+    auto trial = [&](const LaunchTune& t) {
+      fit_ranges(b, recs, t);
+      std::vector<long long> key(1, t.var[a]);
+      for (const LaunchRec& L : recs) key.push_back(L.range);
+      if (std::find(seen.begin(), seen.end(), key) != seen.end()) return;
+      seen.push_back(key);
       cudaError_t ce = cudaSuccess;
-      if (reps > 1 || var != 0 || best == 1e30f) ce = launch_slot(b, recs, b->cur);
+      if (reps > 1 || t.var[a] != 0 || best == 1e30f) ce = launch_slot(b, recs, b->cur);
       float ms = 0;
       while (ce == cudaSuccess) {
         ce = cudaEventRecord(e0, b->stream);
@@ -658,15 +680,32 @@ shasta_status autotune(shasta_batch* b) {
         st = cuda_fail(b, ce, "autotune");
       } else if (ms < best) {
         best = ms;
-        bv = var;
-        bsh = sh;
+        pick = t;
       }
     };
-    for (double sh : shares)
-      if (st == SHASTA_OK) trial(0, sh);
-    if (st == SHASTA_OK) trial(1, bsh);
-    b->tune_var[a] = bv;
-    b->tune_share[a] = bsh;
+    LaunchTune t = b->tune;
+    t.var[a] = 0;
+    if (!in_step) {
+      trial(t);
+    } else if (recs.size() > 1) {
+      for (double sh : pairs)
+        if (st == SHASTA_OK) {
+          t.pair[a] = sh;
+          trial(t);
+        }
+    } else {
+      for (double sh : shares)
+        if (st == SHASTA_OK) {
+          t.share[a] = sh;
+          trial(t);
+        }
+    }
+    if (st == SHASTA_OK) {
+      t = pick;
+      t.var[a] = 1;
+      trial(t);
+    }
+    b->tune = pick;
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);

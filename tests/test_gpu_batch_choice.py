@@ -79,3 +79,42 @@ def test_long_lines_are_cut_beside_other_launches(monkeypatch, shape, count, ahe
             us.append(us_per_step(b))
     assert same(*res)
     assert us[1] < 0.8 * us[0], us
+
+
+def test_two_equations_of_state_are_tuned():
+    """The autotuner times launches that differ for two equations of state side
+    by side: two flat events (measured: 771 us a step with the ranges it picks,
+    913 by the untimed rule, 854 with the other register variant alone), with
+    the same bits."""
+    require_gpu()
+    shape = (500, 500, 30)
+    events = [(shape, eos, 0) for eos in ("ideal", "bag")]
+    pr = [prims(shape, i) for i in range(2)]
+    res, us = [], []
+    for tune in (True, False):
+        with S.Batch(2 * int(np.prod(shape)) + 128, autotune=tune) as b:
+            ids = [b.add_primitives(sh, p, eos=eos) for (sh, eos, _), p in zip(events, pr)]
+            b.step(1)
+            res.append(([b.get_conserved(i) for i in ids], [b.counters(i) for i in ids]))
+            us.append(us_per_step(b))
+    assert same(*res)
+    assert us[0] < 0.9 * us[1], us
+
+
+def test_phases_apart_skip_the_shares():
+    """With events at different phases no share of the trials is used, so only
+    the two register variants are timed: of sweeps over 0.2 ms four an axis, about
+    four steps (eight with the shares)."""
+    require_gpu()
+    shape, ratio = (224, 224, 224), []
+    with S.Batch(3 * 224 ** 3 + 192, autotune=False) as b:
+        for i in range(3):
+            b.add_primitives(shape, prims(shape, i))
+            b.step(1)
+        step = us_per_step(b)
+        for _ in range(5):
+            t = time.perf_counter()
+            b.autotune()
+            b.sync()
+            ratio.append((time.perf_counter() - t) * 1e6 / step)
+    assert min(ratio) < 5.5, ratio
