@@ -38,3 +38,23 @@ def test_thin_grids(monkeypatch, precision, shape, thin):
             assert ranges[thin] >= 24 > shape[thin]
         if thin is None:
             assert all(r <= n for r, n in zip(ranges, shape))
+
+
+@pytest.mark.parametrize("shape,axis,tile", [((300, 20, 24), 0, 100), ((430, 9, 12), 0, 144), ((20, 160, 24), 1, 80),
+                                             ((24, 20, 230), 2, 115)])
+def test_small_grids_show_their_tiles(monkeypatch, shape, axis, tile):
+    """The range of a tiled axis is the length of its tiles (a line in equal
+    parts), which no streamed choice is: those are whole lines or the positions
+    per resident warp, 24 on grids this small."""
+    require_gpu()
+    pr = W.random_state(shape, seed=5, vmax=0.5)
+    U = oracle().prim2cons(OR.params(shape), *pr.as_list())
+    res = []
+    for env in ("", "off"):
+        monkeypatch.setenv("SHASTA_TILE", env)
+        for tune in (False, True):
+            res.append(run(shape, U, tune))
+            assert (res[-1][1][axis] == tile) == (env == ""), (env, tune, res[-1][1])
+    for got, _ in res[1:]:
+        for a, b in zip(res[0][0], got):
+            assert np.array_equal(a, b)
