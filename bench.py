@@ -111,11 +111,18 @@ def measured_peak():
         return FALLBACK_HBM_GBS, "fallback"
 
 
+def kernel_sources():
+    """The sources the sweep kernels are compiled from: their units and every header."""
+    d = os.path.join(ROOT, "paper_1206_0919_gb300", "csrc")
+    return [os.path.join(d, f) for f in sorted(os.listdir(d))
+            if f.endswith((".cuh", ".h")) or (f.endswith(".cu") and f.startswith(("sweep", "tile")))]
+
+
 def kernel_source_hash():
     h = hashlib.sha256()
-    for f in ("sweep.cuh", "sweep_fast.cuh", "sweep_launch.cuh", "sweep_f32.cu",
-              "sweep_mixed.cu", "sweep_f64.cu", "sweep_tile.cuh", "tile_plan.h"):
-        with open(os.path.join(ROOT, "paper_1206_0919_gb300", "csrc", f), "rb") as fh:
+    for f in kernel_sources():
+        h.update(os.path.basename(f).encode())
+        with open(f, "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
 
