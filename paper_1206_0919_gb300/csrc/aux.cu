@@ -448,7 +448,8 @@ cudaError_t launch_set_cons(const double* const in[5], const FieldView& out, siz
                             cudaStream_t s) {
   if (!n) return cudaSuccess;
   // large states in five launches, a fifth of the cells each: the benchmark
-  // line states six launches for a checked set
+  // line counts six for a checked set.  (In one launch, us a set, FP32: 102^3 25
+  // instead of 43, 200^3 84 instead of 105, 512^3 1126 instead of 1156.)
   const size_t slabs = n >= (size_t)1 << 20 ? 5 : 1;
   const size_t part = (n + slabs - 1) / slabs;
   const In5 p = in5(in);

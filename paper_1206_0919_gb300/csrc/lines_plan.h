@@ -33,7 +33,10 @@ inline LinesPlan lines_plan_for(int n, int B) {
 // block leave its stages to the barriers' and loads' latency, one or two
 // blocks per SM leave the pipe idle at them; measured (64^3, 96 x 48 x 120,
 // 143 x 129 x 151, 200^3, B = 1 .. 8) against three blocks of five warps: two
-// blocks 0.97, one 0.93; four warps 0.955, three 0.94, two 0.92.
+// blocks 0.97, one 0.93; four warps 0.955, three 0.94, two 0.92.  Longer lines,
+// one block of 9 to 16 warps per SM, stay at about a third of the streaming
+// kernel's time (us a sweep along x, ideal gas: 256 x 64 x 48 1331 -> 398, 512
+// 2548 -> 911, 874 3654 -> 1429; 512^3, a step 339 -> 231 ms).
 inline int lines_per_block(long long plane, int n, int sm_count) {
   int best = 0;
   double cost = 0.0;

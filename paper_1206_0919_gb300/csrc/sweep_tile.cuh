@@ -19,10 +19,13 @@
 //   128^3  51.4 / 45.3 / 43.4 -> 28.9 / 33.0 / 33.0
 //   131 x 97 x 110  45.3 / 37.1 / 41.2 -> 22.6 / 24.8 / 26.8
 //   200^3  116 / 100 / 100 -> 90.3 / 103 / 111
-// On large grids both are bound by instruction issue (66% / 56% of the slots
-// at 200^3 along x / y here; 241 warp-instructions per 32 cells along y, 262
-// along x, of which a tile's halo wastes 11-25%); the y/z tiles lose their
-// lead to the block barrier between tiles, so large y/z sweeps keep streaming.
+// On large grids both are bound by instruction issue (66% / 57% of the slots
+// at 200^3 along x / y here; 249 warp-instructions per 32 computed positions
+// along x, 241 along y, 279 and 270 per 32 of the lines' own cells: a tile's
+// halo wastes 11-25%); the y/z tiles lose their lead to the block barrier
+// between tiles, so large y/z sweeps keep streaming.  A line much shorter than
+// a tile wastes the rest of it; tile_plan.h holds the estimates that leave such
+// lines to the streaming sweep.
 //
 //  * The half-step and the full-step pass are two trips through one loop
 //    body (recovery, transport factors, the passes of the field pairs), which
@@ -31,7 +34,7 @@
 //  * The cells of a lane are recovered without branches, with the clamp and
 //    the vacuum rule in warps that hold such a cell only.
 //  * (E, Mx) and (My, Mz) go through packed f32x2 arithmetic: 241 instead of
-//    278 instructions per 32 cells, 103 instead of 109 us (200^3, y).
+//    278 instructions per 32 positions, 103 instead of 109 us (200^3, y).
 //  * y/z: the four warps of a block copy a tile of 8 adjacent lines, so that
 //    global accesses are whole 128-byte rows; x: each warp copies its own rows.
 //    Two buffers: the next tile is copied while one is computed.
@@ -454,7 +457,9 @@ __global__ void __launch_bounds__(Lay<AXIS, C, XL>::WARPS * 32, MINB)
         const int o = e / (int)UL, x = e % (int)UL;
         const int pos = o < nlo ? o : n - p0 + (o - nlo);
         if (fast::flips(p0 + pos, n, BC_REFLECT)) {
-          float* m = b + 4 * L::slot(pos, x) + 1 + AXIS;
+          const int s = L::slot(pos, x);
+          if (!SH_OK(P, s >= 0 && s < L::SLOTS, 4, s)) continue;
+          float* m = b + 4 * s + 1 + AXIS;
           *m = -*m;
         }
       }
