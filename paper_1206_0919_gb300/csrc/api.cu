@@ -393,7 +393,7 @@ long long stream_share(const shasta_ctx* c, int axis) {
 // take less than kTileSure of the streamed time.  (A step on 512 x 512 x 4
 // cells, us: tiles 247, streamed 127; on 512 x 512 x 1 228 and 103.)
 constexpr long long kTileAlways = 40, kTileShare = 64;
-constexpr double kTileSure = 0.7;
+constexpr double kTileSure = 0.85;
 
 bool tile_rule(const shasta_ctx* c, int axis, bool sure) {
   const int n = axis == 0 ? c->g.nx : (axis == 1 ? c->g.ny : c->g.nz);
