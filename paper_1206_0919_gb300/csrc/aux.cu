@@ -52,6 +52,24 @@ struct Out6 {
   double* f[6];
 };
 
+// The fields of cell i that `out` asks for (FP32: the quad where any of its four
+// is): a get of one field reads 16 or 4 bytes of a float cell and 8 of a double
+// one, not all of it (320^3, one field of FP64 235 -> 97 us; E of FP32 287 -> 127,
+// R 286 -> 79; all five 327 -> 299).
+__device__ __forceinline__ Cell<float> load_some(const FieldView& f, const Out6& out, size_t i, float) {
+  float4 q = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+  float r = 0.0f;
+  if (out.f[0] || out.f[1] || out.f[2] || out.f[3]) q = static_cast<const float4*>(f.p[0])[i];
+  if (out.f[4]) r = static_cast<const float*>(f.p[4])[i];
+  return Cell<float>{{q.x, q.y, q.z, q.w, r}};
+}
+__device__ __forceinline__ Cell<double> load_some(const FieldView& f, const Out6& out, size_t i, double) {
+  Cell<double> c;
+#pragma unroll
+  for (int k = 0; k < 5; ++k) c.v[k] = out.f[k] ? static_cast<const double*>(f.p[k])[i] : 0.0;
+  return c;
+}
+
 // Conversions between the caller's five arrays and a state, all fields of a
 // cell at once.  Bound by memory: one pass over 60 (FP32) or 80 (FP64) bytes
 // per cell; field by field, the quads were rewritten (or re-read) four times
@@ -80,13 +98,16 @@ __global__ void __launch_bounds__(kThreads) k_get_cons(FieldView in, Out6 out, s
   Cell<T> c[kCells];
 #pragma unroll
   for (int u = 0; u < kCells; ++u)
-    if (i0 + u * kThreads < n) c[u] = load_cell(in, i0 + u * kThreads, T());
+    if (i0 + u * kThreads < n) c[u] = load_some(in, out, i0 + u * kThreads, T());
+  // (widened by the bit patterns: conversion instructions go through the double
+  // pipe, and predicated off they still take their slots)
 #pragma unroll
-  for (int u = 0; u < kCells; ++u)
-    if (i0 + u * kThreads < n)
+  for (int k = 0; k < 5; ++k)
+    if (out.f[k]) {
 #pragma unroll
-      for (int k = 0; k < 5; ++k)
-        if (out.f[k]) out.f[k][i0 + u * kThreads] = double(c[u].v[k]);
+      for (int u = 0; u < kCells; ++u)
+        if (i0 + u * kThreads < n) out.f[k][i0 + u * kThreads] = f64::widen(c[u].v[k]);
+    }
 }
 
 __device__ __forceinline__ double eos_p(const EosParams& q, double e) {
