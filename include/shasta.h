@@ -196,7 +196,8 @@ shasta_status shasta_sweep(shasta_ctx* ctx, int axis);
 
 /* Times the launch choices of the sweep kernels for this grid and keeps the
  * fastest per axis.  FP32 / MIXED: the tiled sweep (short independent pieces
- * of each line; the only choice on small grids; the environment may set
+ * of each line; the only choice on small grids whose lines fill a tile; the
+ * environment may set
  * SHASTA_TILE=off, or the number of a tile shape), or the streaming sweep with
  * a work range length and register variant (a
  * sweep's positions, line groups of 32 lines x positions along the axis, are

@@ -5,7 +5,8 @@
 // throughput on Blackwell:
 //
 // Large grids and batches run it; single contexts take sweep_tile.cuh (the
-// same bits) along x and on grids with too few positions per warp (api.cu).
+// same bits) along x and on grids with too few positions per warp, short lines
+// that would fill little of a tile excepted (api.cu, tile_plan.h).
 //
 //  * State layout: (E, Mx, My, Mz) as one 16-byte quad per cell and R as a
 //    separate array.  A cell moves with one 16-byte and one 4-byte access,
