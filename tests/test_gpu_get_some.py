@@ -1,7 +1,7 @@
 """Getting some of the conserved fields: the bits of a full get, the arrays left
 out untouched, and the time of the fields asked for (one field of five read
-and written: a fifth of the bytes, a third where the float quads are read whole;
-the bound is half)."""
+and written: a fifth of an FP64 get's bytes, two fifths of a float one's, whose
+quads are read whole; the bounds leave half and a fifth for the call itself)."""
 import time
 
 import pytest
@@ -12,8 +12,8 @@ from gpu_util import require_gpu
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("precision", ["fp32", "fp64"])
-def test_single_fields_cost_a_single_field(precision):
+@pytest.mark.parametrize("precision,bound", [("fp32", 0.6), ("fp64", 0.5)])
+def test_single_fields_cost_a_single_field(precision, bound):
     require_gpu()
     import torch
     n = 288
@@ -39,4 +39,4 @@ def test_single_fields_cost_a_single_field(precision):
             one = us([out[j] if j == k else None for j in range(5)])
             assert torch.equal(out[k], full[k])
             assert all(bool((out[j] == -7.0).all()) for j in range(5) if j != k)
-            assert one < 0.5 * whole, (k, one, whole)
+            assert one < bound * whole, (k, one, whole)
